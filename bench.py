@@ -126,11 +126,11 @@ def algo_bytes(kernel, K, mixed):
 # bench command (dram__bytes_read.sum + dram__bytes_write.sum), per particle.  The records
 # hold only while the sources the measured kernels compile from (their files and the shared
 # headers) have the content they had at the capture.
-TRAFFIC_CSRC_SHA256 = "1cee01f75e8560e8e8e3c027c926c2417346d94da4c0722d7aa176479ea4aa51"
+TRAFFIC_CSRC_SHA256 = "cd064e7b83e3f1bc2c8b5ece94c95535d3f3548d4cb42d8106ab6354365ac057"
 TRAFFIC = {
-    "knn": {"workload": "disk22", "bytes_per_particle": 392.34},
-    "rates": {"workload": "disk22", "bytes_per_particle": 196.20},
-    "sample": {"workload": "disk22", "bytes_per_particle": 161.97},
+    "knn": {"workload": "disk22", "bytes_per_particle": 254.56},
+    "rates": {"workload": "disk22", "bytes_per_particle": 189.50},
+    "sample": {"workload": "disk22", "bytes_per_particle": 150.28},
 }
 
 
@@ -139,16 +139,16 @@ TRAFFIC = {
 # warp instructions on the FP64 pipe), under the same source digest rule as TRAFFIC.
 INST_CSRC_SHA256 = TRAFFIC_CSRC_SHA256
 INST = {
-    "knn": {"workload": "disk22", "inst": 654.53, "fp64_inst": 2.0289},
-    "rates": {"workload": "disk22", "inst": 321.52, "fp64_inst": 0.18779},
-    "sample": {"workload": "disk22", "inst": 291.51, "fp64_inst": 6.8512},
+    "knn": {"workload": "disk22", "inst": 439.58, "fp64_inst": 1.8243},
+    "rates": {"workload": "disk22", "inst": 321.47, "fp64_inst": 0.18782},
+    "sample": {"workload": "disk22", "inst": 291.33, "fp64_inst": 6.8355},
 }
 
 # Issue rate of the SMs: 4 schedulers per SM, one warp instruction each per cycle.
 SCHEDULERS_PER_SM = 4
 
 
-KERNEL_SOURCES = ("gd_common.cuh", "gd_ctx.h", "gd_physics.cuh", "k_cells.cu", "k_knn.cu", "k_mc.cu")
+KERNEL_SOURCES = ("gd_common.cuh", "gd_ctx.h", "gd_physics.cuh", "k_tree.cu", "k_knn.cu", "k_mc.cu")
 
 
 def csrc_digest():

@@ -5,7 +5,7 @@
  * of the representative-particle Monte Carlo of "GameDev: GPU-accelerated
  * model for dust evolution" (Sect. 2.5):
  *
- *   gd_build_neighbors    K nearest neighbours over a device cell list,
+ *   gd_build_neighbors    K nearest neighbours over a device search tree,
  *                         sampling measures                      (Sect. 2.5.1)
  *   gd_collision_rates    pair rates lambda_ij = n_ij K_ij, outcome channels,
  *                         controller-bin moments and the executed interval
@@ -27,7 +27,7 @@
  *    data is a DEVICE pointer owned by the caller, who must keep it alive for
  *    the life of the context; the library reads and writes it in place
  *    (s, and x, y, z, vr, lth, lph in gd_push_staggered) and never writes M.
- *  - The library owns its scratch (cell lists, neighbour lists in cell order,
+ *  - The library owns its scratch (search tree, neighbour lists in curve order,
  *    frozen snapshots, controller bins, per-instance state); gd_create
  *    allocates it with cudaMalloc, gd_destroy frees it.
  *  - Every call except gd_stats and gd_destroy only enqueues work on the
@@ -93,7 +93,7 @@ enum {
   GD_ST_DT_FLOOR = 1 << 1,   /* requested interval below dt_coll / 2^60          */
   GD_ST_NONFINITE = 1 << 2,  /* NaN or infinite rate                             */
   GD_ST_KNN = 1 << 3,        /* neighbour search could not find K-1 others       */
-  GD_ST_CAPACITY = 1 << 4,   /* cell grid exceeded its capacity                  */
+  GD_ST_CAPACITY = 1 << 4,   /* an explicit cell size asks for too large a grid  */
   GD_ST_TIMEOUT = 1 << 5     /* a bounded device wait gave up                    */
 };
 
@@ -129,7 +129,9 @@ typedef struct {
   double R_in, R_out;  /* global disk radial edges [cm] (flat-boundary caps)  */
   double box_x, box_y; /* patch periodic extents [cm]                        */
   double t0, m0;       /* test-kernel unit time and mass                     */
-  double cell_size;    /* cell edge [cm]; <= 0: chosen from the data          */
+  double cell_size;    /* cell edge [cm], <= 0: none.  The search tree needs no cells; an
+                          edge whose grid would exceed the library's capacity is
+                          reported (GD_ST_CAPACITY), the lists staying exact     */
   uint64_t seed;       /* Philox key of the instance                         */
   int32_t diff_mode;   /* gd_diffuse: GD_DIFF_PHYSICAL, D = nu/(Sc (1+St^2))
                           with nu = alpha c_s H_g (Sect. 2.4); GD_DIFF_RING, the
@@ -185,10 +187,8 @@ typedef struct {
   double* lph;                 /* DEVICE [N] or NULL: l_phi    (push only)    */
   void* stream;                /* cudaStream_t; NULL = legacy default stream  */
   int64_t max_events_per_interval;   /* per particle; <= 0: 65536              */
-  double cell_factor;          /* cell edge = factor (V_box/N)^(1/3) when the
-                                  instance gives none; <= 0: 1                 */
-  int32_t cell_xsplit;         /* cell x edge = the y/z edge divided by 1, 2 or 4;
-                                  0: 1                                         */
+  double cell_factor;          /* accepted as before, without effect on the search  */
+  int32_t cell_xsplit;         /* 1, 2 or 4 (0: 1), likewise                        */
   int32_t pad1;
 } gd_config;
 
@@ -205,7 +205,7 @@ typedef struct {
   uint32_t status;             /* OR of every instance's GD_ST_* bits          */
   int32_t n_instances;
   double kernel_ms[8];         /* GD_FLAG_TIMING: summed kernel time by step:
-                                  0 cells, 1 knn, 2 rates, 3 interval, 4 sample,
+                                  0 cells (order and tree), 1 knn, 2 rates, 3 interval, 4 sample,
                                   5 push, 6 stats/other, 7 diffusion           */
   int64_t kernel_calls[8];     /* launches timed in each slot                  */
   int64_t knn_redo;            /* mixed form: neighbour searches the FP32 keys
@@ -256,8 +256,8 @@ gd_status gd_create(gd_ctx** out, const gd_config* cfg);
  * service of the library; the paper has no counterpart). */
 gd_status gd_destroy(gd_ctx* ctx);
 
-/* Sect. 2.5.1: bins every particle into a per-instance uniform cell grid
- * (counting sort by cell), then finds each particle's N_K nearest particles
+/* Sect. 2.5.1: sorts every instance's particles along a Hilbert curve, boxes
+ * them into a search tree, then finds each particle's N_K nearest particles
  * of its instance, itself included at zero distance (minimum image across a
  * patch's periodic edges), ranked by (d^2, index) with
  * d^2 = (dx dx + dy dy) + dz dz in FP64.  Lists hold the particle itself in
@@ -500,15 +500,10 @@ gd_status gd_group_stats(gd_ctx* ctx, int32_t instance, int32_t group, gd_group_
  * interval is a round.  Asynchronous. */
 gd_status gd_run_intervals(gd_ctx* ctx, int32_t n, int32_t push);
 
-/* Autotuner: times the cell binning and neighbour search (gd_build_neighbors'
- * kernels) on the current positions for a set of cell shapes -- the y and z edge
- * is factor * (V_box / N)^(1/3) for factor in {0.5, 0.6, 0.7, 0.8, 1.0, 1.2, 1.4},
- * the x edge that divided by 1, 2 or 4 -- with CUDA events, and keeps the fastest
- * for the context (instances with an explicit cell_size keep their edge).  Results never depend on the choice: the lists
- * are exact for any cell size.  Synchronises the stream; call it before
- * gd_run_intervals captures its graph.  Leaves the context ready for
- * gd_build_neighbors.  factor_out, xsplit_out: HOST or NULL, receive the chosen
- * factor and x division. */
+/* Cell shape of the neighbour search.  The search tree adapts to the particles and has no
+ * cell shape to choose, so the call reports the plain one (factor 1, x division 1), drops
+ * a captured graph and waits for the stream.  Leaves the context ready for
+ * gd_build_neighbors.  factor_out, xsplit_out: HOST or NULL. */
 gd_status gd_autotune(gd_ctx* ctx, double* factor_out, int32_t* xsplit_out);
 
 /* Static string for a gd_status code. */

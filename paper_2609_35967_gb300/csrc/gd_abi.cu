@@ -63,9 +63,9 @@ static cudaError_t dalloc(T** p, size_t n) {
 }
 
 static void free_all(gd_ctx* c) {
-  void* ptrs[] = {c->d_off, c->d_tile_off, c->d_inst, c->d_grid, c->d_state, c->d_bins, c->d_cell_count,
-                  c->d_cell_start, c->d_scan_tmp, c->d_cell_of, c->d_slot, c->d_perm, c->d_rank_of,
-                  c->d_pos64, c->d_pos32, c->d_snap64, c->d_snap32, c->d_Mr, c->d_dist, c->d_V,
+  void* ptrs[] = {c->d_off, c->d_tile_off, c->d_inst, c->d_tree, c->d_state, c->d_bins, c->d_stile_off,
+                  c->d_kv[0], c->d_kv[1], c->d_digits, c->d_chunk, c->d_lev, c->d_node_a, c->d_node_b, c->d_perm,
+                  c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64, c->d_snap32, c->d_Mr, c->d_dist, c->d_V,
                   c->d_lam, c->d_nbr, c->d_counters, c->d_sums, c->d_dprev, c->d_redo, c->d_gx,
                   c->d_pref32, c->d_contrib, c->d_MJ, c->d_part, c->d_heavy, c->d_unit_i, c->d_unit_r, c->d_gperm,
                   c->d_uoff, c->d_utile_off, c->d_unit_inst, c->d_tcount, c->d_tbase, c->d_sb, c->d_rperm, c->d_act, c->d_aoff,
@@ -191,7 +191,7 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
     return GD_ERR_CUDA;
   }
 
-  std::vector<long long> tiles = tile_table(c->h_off);
+  std::vector<long long> tiles = tile_table(c->h_off, kTile);
   c->n_tiles = (int)tiles.back();
   // units: one per spatial group of each instance
   c->h_unit0.resize(n);
@@ -205,25 +205,30 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   c->U = (int)unit_inst.size();
   c->n_btiles = c->grouped ? c->n_tiles + c->U : c->n_tiles;
   c->cell_cap = 16 * N + 64LL * n + 1024;
-  long long nst = (c->cell_cap + 2048) / 2048 + 1;   // scan tiles of cells [0, cell_cap]
+  for (int b = 0; b < n; ++b)
+    if (cfg->params[b].cell_size > 0.0) c->check_cells = true;
+  if (c->cell_factor < 1e-3) c->check_cells = true;
+  const std::vector<long long> stiles = tree_plan(c);
 
   bool ok = true;
   ok &= dalloc(&c->d_off, n + 1) == cudaSuccess;
   ok &= dalloc(&c->d_tile_off, n + 1) == cudaSuccess;
   ok &= dalloc(&c->d_inst, n) == cudaSuccess;
-  ok &= dalloc(&c->d_grid, n) == cudaSuccess;
+  ok &= dalloc(&c->d_tree, n) == cudaSuccess;
   ok &= dalloc(&c->d_state, c->U) == cudaSuccess;
   ok &= dalloc(&c->d_bins, c->U) == cudaSuccess;
-  ok &= dalloc(&c->d_cell_count, c->cell_cap + 1) == cudaSuccess;
-  ok &= dalloc(&c->d_cell_start, c->cell_cap + 1) == cudaSuccess;
-  ok &= dalloc(&c->d_scan_tmp, nst) == cudaSuccess;
-  ok &= dalloc(&c->d_cell_of, N) == cudaSuccess;
-  ok &= dalloc(&c->d_slot, N) == cudaSuccess;
+  ok &= dalloc(&c->d_stile_off, n + 1) == cudaSuccess;
+  for (int k = 0; k < 2; ++k) ok &= dalloc(&c->d_kv[k], N) == cudaSuccess;
+  ok &= dalloc(&c->d_digits, 256LL * c->n_stiles) == cudaSuccess;
+  ok &= dalloc(&c->d_chunk, (size_t)c->sort_passes * c->n_chunks) == cudaSuccess;
+  ok &= dalloc(&c->d_lev, c->h_lev.size()) == cudaSuccess;
+  ok &= dalloc(&c->d_node_a, c->n_nodes) == cudaSuccess;
+  ok &= dalloc(&c->d_node_b, c->n_nodes) == cudaSuccess;
   ok &= dalloc(&c->d_perm, N) == cudaSuccess;
   ok &= dalloc(&c->d_rank_of, N) == cudaSuccess;
   ok &= dalloc(&c->d_pos64, N) == cudaSuccess;
   ok &= dalloc(&c->d_snap64, N) == cudaSuccess;
-  ok &= dalloc(&c->d_pos32, N) == cudaSuccess;
+  ok &= dalloc(&c->d_posq, N) == cudaSuccess;
   if (c->precision == GD_MIXED) ok &= dalloc(&c->d_snap32, N) == cudaSuccess;
   ok &= dalloc(&c->d_Mr, N) == cudaSuccess;
   ok &= dalloc(&c->d_dist, N) == cudaSuccess;
@@ -305,6 +310,16 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   }
 
   std::vector<InstDev> inst(n);
+  std::vector<TreeDev> tree(n);
+  for (int b = 0; b < n; ++b) {
+    std::memset(&tree[b], 0, sizeof(TreeDev));
+    for (int l = 0; l < c->max_lev; ++l) {
+      const int* tab = c->h_lev.data() + (size_t)l * (n + 1);
+      tree[b].lev_off[l] = tab[b];
+      tree[b].lev_n[l] = tab[b + 1] - tab[b];
+      if (tree[b].lev_n[l] > 0) tree[b].nlev = l + 1;
+    }
+  }
   std::vector<StateDev> st(c->U);
   for (int b = 0; b < n; ++b) {
     const gd_instance_params& p = c->h_params[b];
@@ -356,6 +371,9 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_off, c->h_off.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_tile_off, tiles.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_stile_off, stiles.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_tree, tree.data(), sizeof(TreeDev) * n, cudaMemcpyHostToDevice, str);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_lev, c->h_lev.data(), sizeof(int) * c->h_lev.size(), cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_inst, inst.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_state, st.data(), sizeof(StateDev) * c->U, cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_bins, 0, sizeof(BinsDev) * c->U, str);
@@ -400,7 +418,7 @@ extern "C" gd_status gd_destroy(gd_ctx* c) {
 }
 
 static gd_status do_build(gd_ctx* c, int32_t* nbr_out, double* d_out) {
-  cudaError_t e = launch_cells(c);
+  cudaError_t e = launch_tree(c);
   if (e == cudaSuccess) e = launch_groups(c);
   if (e == cudaSuccess) e = launch_knn(c);
   if (e == cudaSuccess) e = launch_group_inter(c);
@@ -729,44 +747,15 @@ extern "C" gd_status gd_group_stats(gd_ctx* c, int32_t instance, int32_t group, 
 extern "C" gd_status gd_autotune(gd_ctx* c, double* factor_out, int32_t* xsplit_out) {
   if (!c) return GD_ERR_ARG;
   if (c->phase != 0 && c->phase != 1) return GD_ERR_STATE;
-  static const double kFactors[] = {0.5, 0.6, 0.7, 0.8, 1.0, 1.2, 1.4};
-  static const int kSplits[] = {1, 2, 4};
-  const int saved_flags = c->flags;
-  c->flags &= ~GD_FLAG_TIMING;
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess) { c->flags = saved_flags; return GD_ERR_CUDA; }
-  if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); c->flags = saved_flags; return GD_ERR_CUDA; }
-  double best = c->cell_factor;
-  int best_split = c->cell_xsplit;
-  float best_ms = 1e30f;
-  gd_status st = GD_OK;
-  for (int k = 0; k < 21 && st == GD_OK; ++k) {
-    const double f = kFactors[k / 3];
-    c->cell_factor = f;
-    c->cell_xsplit = kSplits[k % 3];
-    cudaError_t e = launch_cells(c);                  // warm-up: grid and lists for this size
-    if (e == cudaSuccess) e = launch_knn(c);
-    if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-    if (e == cudaSuccess) e = launch_cells(c);
-    if (e == cudaSuccess) e = launch_knn(c);
-    if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float ms = 0.0f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    if (e != cudaSuccess) { st = GD_ERR_CUDA; break; }
-    if (ms < best_ms) { best_ms = ms; best = f; best_split = c->cell_xsplit; }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  c->flags = saved_flags;
-  c->cell_factor = best;
-  c->cell_xsplit = best_split;
+  // the tree search has no cell shape to choose: the plain one is reported
+  c->cell_factor = 1.0;
+  c->cell_xsplit = 1;
   c->phase = 0;
-  c->lists_valid = false;      // the ranks changed: the next collision step builds again
+  c->lists_valid = false;
   if (c->graph_exec) { cudaGraphExecDestroy(c->graph_exec); c->graph_exec = nullptr; c->graph_push = -1; }
-  if (factor_out) *factor_out = best;
-  if (xsplit_out) *xsplit_out = best_split;
-  return st;
+  if (factor_out) *factor_out = c->cell_factor;
+  if (xsplit_out) *xsplit_out = c->cell_xsplit;
+  return cuda_err(cudaStreamSynchronize(c->stream));
 }
 
 extern "C" const char* gd_status_string(gd_status code) {

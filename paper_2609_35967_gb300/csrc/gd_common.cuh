@@ -1,15 +1,17 @@
 // gd_common.cuh -- device-side types and helpers shared by the library's kernels.
 //
 // Layout in HBM (library-owned, one context):
-//   rank space  : particles sorted by (instance, cell); rank r of instance b lies in
-//                 [off[b], off[b+1]) like the caller's indices.  perm[r] is the caller
-//                 index, rank_of[i] its inverse.
-//   Pos64[r]    : {x, y, z, caller index}            32 B  (FP64 K-NN, re-rank)
-//   float4 pos32: {x, y, z relative to the own cell origin, packed cell (11+11+10 bits)} 16 B
+//   rank space  : particles of an instance sorted along a Hilbert curve (equal keys by caller
+//                 index); rank r of instance b lies in [off[b], off[b+1]) like the caller's
+//                 indices.  perm[r] is the caller index, rank_of[i] its inverse.
+//   int4 posq   : {x, y, z in units of the instance's quantum, caller index (~index when a
+//                 coordinate is not finite)}                          16 B  (K-NN candidates)
+//   Pos64[r]    : {x, y, z, caller index}            32 B  (exact keys, gas at the particle)
+//   nodes       : bounding boxes of 32 consecutive ranks (leaves), of 32 leaves, ... up to a
+//                 level of at most 32 nodes per instance             24 B per node
 //   Snap64[r]   : {s, m, N, 1/m} frozen at the interval start        32 B
 //   float4 snap32: {s, m, N 2^-64, 1/m} frozen, FP32                 16 B
 //   nbr[r*K+k]  : ranks of the K neighbours, slot 0 = self, others by ascending caller index
-//   cell_start  : exclusive scan of per-cell counts, instance grids concatenated
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -109,20 +111,21 @@ __device__ __forceinline__ int group_of(const InstDev& p, double x, double y) {
   return (int)f;
 }
 
-// Uniform cell grid of one instance, rebuilt every interval from the data bounds.
-struct GridDev {
+// The search tree of one instance.  The frame (origin, quantum, periodic extents) is rebuilt
+// from the data bounds at every build; the levels' extents follow from the particle count.
+constexpr int kLeaf = 32;        // ranks per leaf and children per node
+constexpr int kMaxLev = 6;       // 2^31 particles: 2^26 leaves, 2^21, 2^16, 2^11, 2^6, 2
+struct TreeDev {
   double lo[3];      // origin
-  double cs[3];      // cell edge per axis
-  double inv[3];     // 1 / cs
-  double box[3];     // periodic extent (x, y of a patch), 0 otherwise
-  double ctr[3];     // origin of the FP32 mirror coordinates
-  double X32;        // bound on |coordinate| + periodic extents (FP64 rounding of the mirror)
-  float cs32[3];     // cell edges and their inverses in FP32 (search bookkeeping)
-  float inv32[3];
-  float E32;         // absolute error bound of FP32 cell-relative distances [cm]
-  int dim[3];
-  int periodic;      // x and y periodic (patch)
-  long long cell_off;
+  double q, inv_q;   // quantum [cm per unit] of all axes and its inverse
+  double box[2];     // periodic extents of x and y (patch), 0 otherwise
+  int boxq[2];       // the same in units, rounded
+  int maxq[2];       // largest x and y unit of the data (periodic instances)
+  int periodic;
+  int bits;          // units fit in this many bits
+  int nlev;          // levels; the top one has at most kLeaf nodes
+  int pad;
+  int lev_off[kMaxLev], lev_n[kMaxLev];   // first node (concatenated levels) and node count
 };
 
 // Mutable per-instance state (device resident).
@@ -230,6 +233,17 @@ __device__ __forceinline__ int inst_of(const long long* __restrict__ off, int n_
   return lo;
 }
 
+// Instance of a node from one level's table of first nodes (an instance without nodes at the
+// level shares its entry with the next).
+__device__ __forceinline__ int lev_inst(const int* __restrict__ tab, int n_inst, int node) {
+  int lo = 0, hi = n_inst - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(&tab[mid]) <= node) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
 // Order-preserving map of doubles to unsigned 64-bit integers (for atomic min/max).
 __device__ __forceinline__ unsigned long long dbl_ord(double v) {
   unsigned long long b = (unsigned long long)__double_as_longlong(v);
@@ -256,20 +270,6 @@ __device__ __forceinline__ int fine_bin(double s) {
   int t = 3 * e + (mb >= e1 ? 1 : 0) + (mb >= e2 ? 1 : 0);
   t -= kTMin;
   return t < 0 ? 0 : (t > kNFine - 1 ? kNFine - 1 : t);
-}
-
-// Cell index of a coordinate along one axis of an instance grid; periodic axes wrap.
-__device__ __forceinline__ int axis_cell(const GridDev& g, int a, double v) {
-  double t = floor((v - g.lo[a]) * g.inv[a]);
-  int d = g.dim[a];
-  if (g.box[a] > 0.0) {
-    t = fmin(fmax(t, -1e15), 1e15);
-    long long k = (long long)t;
-    k %= d;
-    if (k < 0) k += d;
-    return (int)k;
-  }
-  return t < 0.0 ? 0 : (t >= (double)d ? d - 1 : (int)t);
 }
 
 // ---------------------------------------------------------------- Philox4x32-10

@@ -11,9 +11,8 @@ struct gd_ctx {
   // configuration
   int n_inst = 0, K = 0, precision = 0, flags = 0;
   long long N = 0;
-  double cell_factor = 1.0;
-  int cell_xsplit = 1;                  // x cells per cell edge (rows are y-z lines; finer x
-                                        // cells trim each row's x range at no extra row cost)
+  double cell_factor = 1.0;             // accepted and checked; the tree search has no cells
+  int cell_xsplit = 1;
   long long max_events = 65536;
   cudaStream_t stream = nullptr;
   int num_sms = 0;
@@ -32,25 +31,38 @@ struct gd_ctx {
   long long* d_tile_off = nullptr;      // [n_inst + 1] first per-particle tile of each instance
   int n_tiles = 0;
   gd::InstDev* d_inst = nullptr;        // [n_inst]
-  gd::GridDev* d_grid = nullptr;        // [n_inst]
+  gd::TreeDev* d_tree = nullptr;        // [n_inst] search trees
   gd::StateDev* d_state = nullptr;      // [n_inst]
   gd::BinsDev* d_bins = nullptr;        // [n_inst]
-  long long cell_cap = 0;               // capacity of the concatenated cell arrays
-  int* d_cell_count = nullptr;          // [cell_cap + 1]
-  int* d_cell_start = nullptr;          // [cell_cap + 1]
-  int* d_scan_tmp = nullptr;            // block sums of the scan
-  int* d_cell_of = nullptr;             // [N] cell of each caller index
-  int* d_slot = nullptr;                // [N] position inside the cell
+  long long cell_cap = 0;               // bound on the cells an explicit cell size may ask for
+  bool check_cells = false;             // some instance's cell size has to be checked against it
+  // Hilbert order: segmented radix sort of (key, caller index) pairs over tiles of kSortTile
+  int n_stiles = 0;
+  long long* d_stile_off = nullptr;     // [n_inst + 1] first sort tile of each instance
+  int sort_passes = 0;                  // 8-bit digits sorted
+  uint2* d_kv[2] = {nullptr, nullptr};  // [N] pairs, double buffer
+  int* d_digits = nullptr;              // [256 n_stiles] digit counts, then their exclusive scan
+  int* d_chunk = nullptr;               // [sort_passes * n_chunks] sums over chunks of d_digits
+  int n_chunks = 0;
+  // search tree
+  int n_leaves = 0;                     // of all instances
+  int n_nodes = 0;                      // of all levels
+  int max_lev = 1;                      // levels of the deepest instance
+  int* d_lev = nullptr;                 // [kMaxLev * (n_inst + 1)] first node of each instance at
+                                        // each level (absolute; end entry: one past the level)
+  std::vector<int> h_lev;
+  float4* d_node_a = nullptr;           // [n_nodes] box {lo x, lo y, lo z, hi x} in units
+  float2* d_node_b = nullptr;           // [n_nodes] {hi y, hi z}
   int* d_perm = nullptr;                // [N] rank -> caller index
   int* d_rank_of = nullptr;             // [N] caller index -> rank
   gd::Pos64* d_pos64 = nullptr;         // [N]
-  float4* d_pos32 = nullptr;            // [N]
+  int4* d_posq = nullptr;               // [N] quantised positions and caller index
   gd::Snap64* d_snap64 = nullptr;       // [N]
   float4* d_snap32 = nullptr;           // [N]
   double* d_Mr = nullptr;               // [N] M in rank order
   double* d_dist = nullptr;             // [N] d_i, rank order
   double* d_dprev = nullptr;            // [N] d_i of the last build, caller order (0: none)
-  int* d_redo = nullptr;                // [N] mixed K-NN: queries the FP64 form redoes
+  int* d_redo = nullptr;                // [N] K-NN: queries redone exactly; mixed rates: ranks redone
   int* d_heavy = nullptr;               // [N] sampler: the particles sampled one per warp first
   double* d_V = nullptr;                // [N] V_i, rank order
   double* d_lam = nullptr;              // [N] lambda*_i, rank order
@@ -120,7 +132,7 @@ struct gd_ctx {
   long long launches = 0;
   long long diff_step = 0;              // gd_diffuse calls so far (Philox counter word 1)
   bool lists_valid = false;             // neighbour lists built (gd_collide may reuse them)
-  bool moved = false;                   // particles moved since the last neighbour build
+  bool moved = true;                    // no previous build, or particles moved since it
 
   // timing
   static constexpr int kSlots = 8;
@@ -157,7 +169,8 @@ inline TileMap bins_map(const gd_ctx* c) {
 }
 
 // launchers (each returns cudaGetLastError() of its launches)
-cudaError_t launch_cells(gd_ctx* c);
+std::vector<long long> tree_plan(gd_ctx* c);   // sort tiles and levels from the offsets
+cudaError_t launch_tree(gd_ctx* c);         // Hilbert order, rank-space copies, search tree
 cudaError_t launch_knn(gd_ctx* c);
 cudaError_t knn_prepare(gd_ctx* c);
 cudaError_t launch_rates(gd_ctx* c, double* chan_out);
@@ -183,7 +196,7 @@ cudaError_t launch_spectrum(gd_ctx* c);
 cudaError_t launch_outputs_knn(gd_ctx* c, int* nbr_out, double* d_out);
 cudaError_t launch_outputs_lam(gd_ctx* c, double* lam_out);
 
-std::vector<long long> tile_table(const std::vector<long long>& off);
+std::vector<long long> tile_table(const std::vector<long long>& off, int tile);
 
 // event timing around a launch (no-op unless GD_FLAG_TIMING)
 void time_begin(gd_ctx* c, int slot);

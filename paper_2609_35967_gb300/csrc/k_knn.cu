@@ -1,28 +1,41 @@
-// k_knn.cu -- K nearest neighbours over the device cell list (Sect. 2.5.1).
+// k_knn.cu -- K nearest neighbours over the Hilbert-ordered tree (Sect. 2.5.1).
 //
-// Lane = query.  Consecutive threads take consecutive query ranks (neighbouring cells),
-// and every thread runs the whole search of its own particle.  The only shared resource
-// is the warp's slice of shared memory, where lane l keeps its candidates: word w of
-// entry e at [(w * CAP + e) * 33 + l], so lanes touching the same entry, or one lane
-// walking its entries, never share a bank.
+// A warp takes one leaf: 32 queries that are consecutive on the curve, lane = query.  Their
+// balls overlap almost wholly, so the warp walks the tree once for all of them, stages the
+// candidates near the leaf's box in shared memory and every lane tests the same candidate at
+// the same time, read by broadcast: no lane waits for another's rows, and a test is a handful
+// of FP32 instructions (two candidates per packed instruction).
 //
-//  radius : 1.001 x the particle's d_i of the previous build when there is one (exact
-//           when the particles did not move; after a push the radius search corrects it),
-//           else an estimate from the particle count of the 27 cells around it;
-//  scan   : the cell rows that meet the ball are produced row by row and consumed
-//           candidate by candidate in one loop (the cell starts of the next row are
-//           loaded while the current row is scanned); keys inside the ball are kept;
-//  radius : grows or shrinks (bisection between radii known to hold too few / too many
-//           candidates) until the ball holds between K-1 and CAP other particles;
-//  keys   : FP64 form -- d^2 = (dx dx + dy dy) + dz dz in FP64 (no FMA, minimum image),
-//           ties by caller index: the oracle's order exactly.
-//           Mixed form -- FP32 D from cell-relative FP32 coordinates, ties by rank; with
-//           |sqrt(D) - d| <= 10u sqrt(D) + E (u = 2^-24) keys below T_lo are certain
-//           members and keys up to T_hi form a band ranked exactly in FP64.  A band wider
-//           than kBand, a periodic axis covered whole, or no acceptable radius puts the
-//           query on a list that the FP64 form then redoes.
-//  output : d_i = sqrt of the (K-1)-th d^2, V_i with the flat-boundary caps, and the row:
-//           the particle itself, then its members by ascending caller index.
+//  find   : the leaves whose box comes within the largest radius of the queries' box, level by
+//           level, lane = child, four nodes at a time;
+//  visit  : four of these leaves' particles are loaded at a time (lane = particle), those within
+//           the radius of the queries' box are queued in shared memory;
+//  test   : every lane tests the same queued candidate at the same time, read by broadcast: FP32
+//           D in units of the instance's quantum, two candidates per packed instruction, a hit
+//           appended to the lane's list under a predicate;
+//  decide : |sqrt(D) - d| <= 10u sqrt(D) + E (u = 2^-24) separates certain members from a band
+//           ranked exactly in FP64 by (d^2, caller index), d^2 = (dx dx + dy dy) + dz dz (no
+//           FMA, minimum image).  The lists are the exact FP64 ones in both forms;
+//  output : d_i = sqrt of the (K-1)-th d^2, V_i with the flat-boundary caps, and the row: the
+//           particle itself, then its members by ascending caller index.
+//
+// k_knn<., ., true>  (particles that did not move): the radius is the previous build's d_i and a
+//           hair, so the K-1 members and rarely more are hit.  Leaves where that fails for many
+//           queries (no earlier build, or the caller changed the positions) are listed for
+// k_knn<., ., false> (moved particles, first builds and those leaves): the hits go to a buffer of
+//           two to three times the members as words (upper bits of D, place), and the K-1
+//           smallest are chosen.  A query with too few or too many hits walks again with a
+//           rescaled radius; one that stays undecided is listed for
+// k_knn_exact: a warp per query, branch and bound over the tree with FP64 keys (d^2, caller
+//           index) in a list held across the warp's lanes; exact for any ties.
+//
+// Bound by instruction issue and the latency of dependent steps, not by HBM: 437 warp
+// instructions per particle at K = 32 (a uniform cell grid walked by each lane alone took 654,
+// with its lanes waiting for one another), 55% of the issue slots, about 510 candidates tested
+// per leaf of 32 queries.  Builds of a 2^22-particle disk, K = 32: static 5.0 -> 3.6 ms, first
+// 36.6 -> 16 ms; after a push 10.8 -> 6.5 ms (2^20: 2.6 -> 1.6); K = 48 after a push 14.7 -> 8.3
+// ms.  The code is kept small on purpose (loops not unrolled, the reduced models' volume out of
+// line): unrolled, it missed the instruction cache and the same builds took half again as long.
 #include <climits>
 
 #include "gd_ctx.h"
@@ -30,19 +43,36 @@
 
 namespace gd {
 
-constexpr int kBand = 8;          // band entries resolved in FP64 per mixed query
+constexpr int kExtra = 4;         // static: hits beyond the members that are sorted out
+constexpr int kBand = 8;          // band entries resolved in FP64 per query
 constexpr int kPad = 33;          // words per entry row of a warp's buffer (32 lanes + 1)
+constexpr int kQueue = 160;       // candidates staged: what is left over and four leaves
+constexpr uint32_t kPlaceMask = 8191u;
+constexpr int kSlack = 8;
+constexpr int kSlots = 256;       // leaves one walk may reach (8 + 5 bits of a candidate's place)
+constexpr int kFront = 64;        // nodes of an upper level one walk may reach
+constexpr int kShiftBit = 26;     // an instance's leaves fit below (2^31 particles)
+constexpr int kMaxWarps = 20;     // warps an SM holds at most, the registers shared among them
+                                  // (16: 4% slower, 24: 5% slower, both by spills or idle slots)
+constexpr int kTries = 6;
+constexpr float kMovedFac = 1.04f;  // after a push: 1.03 to 1.08 within 5% of one another (2^20 disk)
+constexpr float kLeafShare = 0.18f;  // first radius: see k_knn
+constexpr int kOver = 4;          // a lane with more than kOver times its buffer's entries ends its walk
+constexpr float kSplit = 40.0f;   // see k_knn
+constexpr float kRel = 10.0f * 5.9604645e-8f;
+constexpr unsigned kAll = 0xffffffffu;
 
 struct KnnArgs {
   long long N;
-  int K, n_inst;
+  int K, n_inst, n_leaves;
   const long long* off;
+  const int* leaf_off;            // [n_inst + 1] first leaf of each instance
   const InstDev* P;
-  const GridDev* grid;
-  const int* cstart;
+  const TreeDev* tree;
+  const float4* na;               // node boxes
+  const float2* nb;
+  const int4* posq;
   const Pos64* pos64;
-  const float4* pos32;
-  const int* perm;
   const int* rank_of;
   int* nbr;
   double* dist;
@@ -50,151 +80,21 @@ struct KnnArgs {
   float* pref32;                  // mixed form: FP32 rate prefactor (NULL in the FP64 form)
   double* dprev;                  // caller order: d_i of the last build (0: unknown)
   StateDev* st;
-  int* redo;                      // mixed form: queries the FP64 form redoes
+  int* leaves;                    // leaves (and parts of them) with undecided queries (their dist is -1)
+  unsigned long long* leaves_n;
+  int listed;                     // 1: only the listed leaves and their undecided queries
+  int* redo;                      // queries for k_knn_exact
   unsigned long long* redo_n;
-  const int* list;                // FP64 redo pass: the queries to process
-  const unsigned long long* list_n;
-  float rfac;                     // first radius = rfac d_i of the last build
+  int parts;                      // warps a leaf's queries are spread over (1, 2 or 4)
+  int packed;                     // caller indices leave room for a buffer entry in a sort key
 };
 
-// ---------------------------------------------------------------- geometry (FP32 / INT)
-struct QueryPos {
-  double x, y, z;     // FP64 position (FP64 keys)
-  int ix, iy, iz;     // own cell
-  float fx, fy, fz;   // position inside the own cell [cm]
-};
-
-struct Grid32 {
-  float cs[3], inv[3];
-  int dim[3];
-  bool per;           // x and y periodic
-  long long cell_off;
-};
-
-// Conservative cell range [lo, hi] (unwrapped on periodic axes) of the slab
-// |coordinate - query| <= rs along one axis; full = a periodic axis covered whole.
-__device__ __forceinline__ void axis_range32(const Grid32& G, int a, int ia, float fa, float rs, int& lo,
-                                             int& hi, bool& full) {
-  const float m = rs * 1.00001f + G.cs[a] * 1e-5f;
-  float t0 = floorf((fa - m) * G.inv[a]);
-  float t1 = floorf((fa + m) * G.inv[a]);
-  const int d = G.dim[a];
-  t0 = fmaxf(t0, -4.0e6f);
-  t1 = fminf(t1, 4.0e6f);
-  lo = ia + (int)t0;
-  hi = ia + (int)t1;
-  full = false;
-  if (G.per && a < 2) {
-    if (hi - lo + 1 >= d) { lo = 0; hi = d - 1; full = true; }
-  } else {
-    lo = lo < 0 ? 0 : lo;
-    hi = hi > d - 1 ? d - 1 : hi;
-  }
-}
-
-// Lower bound of the distance from the query to the slab of (unwrapped) cell k.
-__device__ __forceinline__ float slab_dist32(const Grid32& G, int a, int ia, float fa, int k) {
-  float d;
-  if (k < ia) d = (float)(ia - k - 1) * G.cs[a] + fa;
-  else if (k > ia) d = (float)(k - ia) * G.cs[a] - fa;
-  else d = 0.0f;
-  return fmaxf(d * 0.99999f - G.cs[a] * 1e-5f, 0.0f);
-}
-
-__device__ __forceinline__ int floordiv(int a, int d) {
-  int q = a / d;
-  return (a % d != 0 && ((a < 0) != (d < 0))) ? q - 1 : q;
-}
-
-// One row segment: cells [ca, cb) of the concatenated cell arrays, the x shift of a
-// periodic wrap (cells) and the row's y and z offsets from the query cell.
-struct Seg {
-  long long ca, cb;
-  int xsh, dyc, dzc;
-};
-
-// Rows (z outer, y inner) of the ball of radius rs around the query, one segment per
-// call (a row wrapped across a periodic x edge gives two).
-struct RowIter {
-  int lz, hz, ly, hy;
-  int iz, iyu;
-  bool fy, pending;
-  float rs2;
-  Seg pend;
-};
-
-__device__ __forceinline__ void rows_begin(const Grid32& G, const QueryPos& Q, float rs, RowIter& it, bool& amb) {
-  bool fz;
-  axis_range32(G, 2, Q.iz, Q.fz, rs, it.lz, it.hz, fz);
-  axis_range32(G, 1, Q.iy, Q.fy, rs, it.ly, it.hy, it.fy);
-  if (it.fy && G.per) amb = true;
-  it.iz = it.lz;
-  it.iyu = it.ly;
-  it.pending = false;
-  it.rs2 = rs * rs * 1.00002f;
-  if (it.hy < it.ly) it.iz = it.hz + 1;   // empty
-}
-
-__device__ __forceinline__ bool rows_next(const Grid32& G, const QueryPos& Q, RowIter& it, Seg& s, bool& amb) {
-  if (it.pending) {
-    it.pending = false;
-    s = it.pend;
-    if (++it.iyu > it.hy) { it.iyu = it.ly; ++it.iz; }
-    return true;
-  }
-  const int dimx = G.dim[0], dimy = G.dim[1];
-  while (it.iz <= it.hz) {
-    const int iz = it.iz, iyu = it.iyu;
-    bool got = false;
-    const float dz = slab_dist32(G, 2, Q.iz, Q.fz, iz);
-    const float dy = it.fy ? 0.0f : slab_dist32(G, 1, Q.iy, Q.fy, iyu);
-    const float dyz2 = dy * dy + dz * dz;
-    if (dyz2 <= it.rs2) {
-      const float xr = sqrtf(fmaxf(it.rs2 - dyz2, 0.0f));
-      int lx, hx;
-      bool fx;
-      axis_range32(G, 0, Q.ix, Q.fx, xr, lx, hx, fx);
-      if (lx <= hx) {
-        if (fx && G.per) amb = true;
-        int iy = iyu;
-        if (G.per) { iy %= dimy; if (iy < 0) iy += dimy; }
-        const long long rowc = G.cell_off + (long long)dimx * (iy + (long long)dimy * iz);
-        int kx = 0, a0 = lx, e0 = hx;
-        if (G.per && !fx) {
-          kx = floordiv(lx, dimx);
-          a0 = lx - kx * dimx;
-          e0 = hx - kx * dimx;
-        }
-        const int e1 = e0 < dimx ? e0 : dimx - 1;
-        s.ca = rowc + a0;
-        s.cb = rowc + e1 + 1;
-        s.xsh = kx * dimx;
-        s.dyc = iyu - Q.iy;
-        s.dzc = iz - Q.iz;
-        if (e0 >= dimx) {
-          it.pending = true;
-          it.pend.ca = rowc;
-          it.pend.cb = rowc + (e0 - dimx) + 1;
-          it.pend.xsh = (kx + 1) * dimx;
-          it.pend.dyc = s.dyc;
-          it.pend.dzc = s.dzc;
-          return true;             // the row advances after its second segment
-        }
-        got = true;
-      }
-    }
-    if (++it.iyu > it.hy) { it.iyu = it.ly; ++it.iz; }
-    if (got) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ double sample_volume_reduced(const InstDev& P, double d, double x, double y);
+__device__ double sample_volume_reduced(const InstDev& P, double d, double x, double y);
 
 __device__ __forceinline__ double sample_volume(const InstDev& P, double d, double x, double y) {
   if (P.kernel_mode != GD_KERNEL_PHYSICAL) return 1.0;
   if (P.model != GD_MODEL_3D) return sample_volume_reduced(P, d, x, y);
-  double V = 4.0 * kPi * d * d * d / 3.0;
+  double V = (4.0 * kPi / 3.0) * d * d * d;
   if (P.geometry == GD_GEOM_DISK) {
     const double R2 = x * x + y * y;
     const double a = P.R_in + d, bo = P.R_out - d;
@@ -215,7 +115,8 @@ __device__ __forceinline__ double sample_volume(const InstDev& P, double d, doub
 // straight line; the 1D annulus [R - d, R + d] clipped at the edges) times 2 pi R (2D
 // radial-polar: a toroidal volume) or times the vertical length sqrt(2 pi (H_i^2 + H_j^2))
 // of the Gaussian average with H_i = H_j = H_g(R_i) (vertically integrated models).
-__device__ __forceinline__ double sample_volume_reduced(const InstDev& P, double d, double x, double y) {
+// Out of line: the gas disk's powers and the arc cosines are 70 KB of code.
+__device__ __noinline__ double sample_volume_reduced(const InstDev& P, double d, double x, double y) {
   double R;
   if (P.geometry == GD_GEOM_PATCH) R = P.r0 + x;
   else if (P.model == GD_MODEL_RPHI) R = __dsqrt_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)));
@@ -239,42 +140,6 @@ __device__ __forceinline__ double sample_volume_reduced(const InstDev& P, double
   return A * sqrt(2.0 * kPi * (g.H * g.H + g.H * g.H));
 }
 
-// Radius estimate from the particle count of the 27 cells around the query.
-__device__ __forceinline__ float rho_start(const Grid32& G, const int* __restrict__ cstart, const QueryPos& Q,
-                                           int L) {
-  int n = 0, nc = 0;
-  for (int c = 0; c < 27; ++c) {
-    const int dx = c % 3 - 1, dy = (c / 3) % 3 - 1, dz = c / 9 - 1;
-    int ix = Q.ix + dx, iy = Q.iy + dy;
-    const int iz = Q.iz + dz;
-    bool ok = iz >= 0 && iz < G.dim[2];
-    if (G.per) {
-      ix %= G.dim[0]; if (ix < 0) ix += G.dim[0];
-      iy %= G.dim[1]; if (iy < 0) iy += G.dim[1];
-    } else {
-      ok = ok && ix >= 0 && ix < G.dim[0] && iy >= 0 && iy < G.dim[1];
-    }
-    if (ok) {
-      const long long cc = G.cell_off + ix + (long long)G.dim[0] * (iy + (long long)G.dim[1] * iz);
-      n += __ldg(&cstart[cc + 1]) - __ldg(&cstart[cc]);
-      nc += 1;
-    }
-  }
-  const float csmax = fmaxf(G.cs[0], fmaxf(G.cs[1], G.cs[2]));
-  if (n <= 1) return 2.0f * csmax;
-  // density in units of csmax^3 (a cell volume in cm^3 can exceed the FP32 range)
-  const float vcell = (G.cs[0] / csmax) * (G.cs[1] / csmax) * (G.cs[2] / csmax);
-  const float nd = (float)(n - 1) / ((float)nc * vcell);
-  const float r = 1.2f * csmax * cbrtf(3.0f * (float)L / (4.0f * 3.14159265f * nd));
-  return fminf(fmaxf(r, 1e-3f * csmax), 4.0f * csmax * (float)(G.dim[0] + G.dim[1] + G.dim[2]));
-}
-
-__device__ __forceinline__ float grow(float rho, int found, int L, int cap) {
-  // few found: the count says little, so grow by at least a quarter
-  const float g = cbrtf(0.5f * (float)(L + cap) / (float)(found > 0 ? found : 1));
-  return rho * fminf(fmaxf(g, 4 * found >= L ? 1.01f : 1.25f), 3.0f);
-}
-
 // Minimum-image FP64 d^2 of rank r from the query: the oracle's expression.
 __device__ __forceinline__ double d2_fp64(const Pos64* __restrict__ pos64, int r, double qx, double qy,
                                           double qz, double bx, double by, long long& j) {
@@ -289,233 +154,372 @@ __device__ __forceinline__ double d2_fp64(const Pos64* __restrict__ pos64, int r
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// ---------------------------------------------------------------- the lane's buffer
-// kMixed: word 0 = bits of the FP32 D, word 1 = rank.  FP64: words 0/1 = low/high bits of
-// d^2, word 2 = caller index.  Entries compare as (key, tie) with unsigned integers
-// (non-negative floats order like their bit patterns).
-template <int CAP, bool kMixed>
-struct LaneBuf {
-  static constexpr int NW = kMixed ? 2 : 3;
-  uint32_t* b;
-  __device__ __forceinline__ uint32_t& w(int word, int e) const { return b[(word * CAP + e) * kPad]; }
-  __device__ __forceinline__ unsigned long long key(int e) const {
-    if (kMixed) return ((unsigned long long)w(0, e) << 32) | w(1, e);
-    return ((unsigned long long)w(1, e) << 32) | w(0, e);
-  }
-  __device__ __forceinline__ void swap(int a, int b2) const {
-#pragma unroll
-    for (int k = 0; k < NW; ++k) { const uint32_t t = w(k, a); w(k, a) = w(k, b2); w(k, b2) = t; }
-  }
-  // Leaves the L smallest of entries [0, n) in [0, L) (any order) by moving the largest
-  // remaining entry to the tail n - L times (the radius keeps n - L small); returns the
-  // index of the largest of them, the L-th smallest.
-  __device__ __forceinline__ int select(int n, int L) const {
-    for (int m = n; m > L; --m) {
-      const int im = argmax(m);
-      if (im != m - 1) swap(im, m - 1);
-    }
-    return argmax(L);
-  }
-  // index of the largest of entries [0, m), the running maximum kept in registers
-  __device__ __forceinline__ int argmax(int m) const {
-    int im = 0;
-    unsigned long long km = key(0);
-    uint32_t jm = kMixed ? 0u : w(2, 0);
-    for (int e = 1; e < m; ++e) {
-      const unsigned long long ke = key(e);
-      if (kMixed) {
-        if (ke > km) { km = ke; im = e; }
-      } else {
-        const uint32_t je = w(2, e);
-        if (ke > km || (ke == km && je > jm)) { km = ke; jm = je; im = e; }
-      }
-    }
-    return im;
-  }
+// Result of one query: d_i, V_i, the rate prefactor and the next build's radius.
+__device__ __forceinline__ void put_result(const KnnArgs& A, const InstDev& P, long long q, int ci, double d2max,
+                                           double x, double y) {
+  const double d = sqrt(d2max);
+  A.dist[q] = d;
+  const double Vq = sample_volume(P, d, x, y);
+  A.V[q] = Vq;
+  if (A.pref32) A.pref32[q] = (float)rate_prefactor(P, Vq, A.K, true);
+  A.dprev[ci] = d;
+}
+
+// Squared distance between two intervals' or a point's and a box's nearest points, per axis.
+__device__ __forceinline__ float gap(float alo, float ahi, float blo, float bhi) {
+  return fmaxf(fmaxf(alo - bhi, blo - ahi), 0.0f);
+}
+
+__device__ __forceinline__ float grow(float rho, int found, int L, int cap) {
+  // few found: the count says little, so grow by at least a quarter
+  const float g = cbrtf(0.5f * (float)(L + cap) / (float)(found > 0 ? found : 1));
+  return rho * fminf(fmaxf(g, 4 * found >= L ? 1.01f : 1.25f), 2.0f);
+}
+
+// Two FP32 values in one register pair and their packed arithmetic (each half rounded like the
+// scalar instruction).
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Candidates of a walk, relative to the queries' box; place: the candidate's leaf (its entry in
+// tab) and lane.
+struct Queue {
+  float x[kQueue + 32], y[kQueue + 32], z[kQueue + 32];   // past kQueue: what is not kept
+  unsigned place[kQueue + 32];
 };
 
-// Candidates of the ball of radius rho; keys inside it go to the buffer (the first CAP of
-// them).  Returns how many were inside.
-// kRow1: a one-row grid (the 1D radial model) packs the x cell in all the bits of w.
-template <int CAP, bool kMixed, bool kRow1>
-__device__ __forceinline__ int scan_ball(const KnnArgs& A, const Grid32& G, const GridDev& Gd, const QueryPos& Q,
-                                         long long q, float rho, const LaneBuf<CAP, kMixed>& buf, bool& amb) {
-  const float rel = 10.0f * 5.9604645e-8f;
-  const float E = Gd.E32;
-  const float rf = (rho * (1.0f + 2.0f * rel) + 2.0f * E) * 1.000001f;
-  const float rhof2 = rf * rf * 1.000001f;
-  const double rho2 = (double)rho * (double)rho;
-  const double bx = Gd.box[0], by = Gd.box[1];
-  const int* __restrict__ cstart = A.cstart;
-  RowIter it;
-  rows_begin(G, Q, rho, it, amb);
-  // rows in order; the cell starts of the next row are loaded before the current row is
-  // scanned.  Neighbouring queries mostly share their rows, so the lanes of a warp walk
-  // the same candidates together.
-  Seg cur, nxt;
-  cur.xsh = cur.dyc = cur.dzc = 0;
-  bool has_cur = rows_next(G, Q, it, cur, amb);
-  int ca = 0, cb = 0;
-  if (has_cur) { ca = __ldg(cstart + cur.ca); cb = __ldg(cstart + cur.cb); }
-  int n_in = 0;
-  while (has_cur) {
-    nxt.xsh = nxt.dyc = nxt.dzc = 0;
-    const bool has_nxt = rows_next(G, Q, it, nxt, amb);
-    int na = 0, nb = 0;
-    if (has_nxt) { na = __ldg(cstart + nxt.ca); nb = __ldg(cstart + nxt.cb); }
-    const float dycf = (float)cur.dyc * G.cs[1], dzcf = (float)cur.dzc * G.cs[2];
-    const int xoff = cur.xsh - Q.ix;
-    if (kMixed) {
-      // four candidates per step, their loads issued together
-      for (int r0 = ca; r0 < cb; r0 += 4) {
-        float4 p[4];
+// The walk's state common to the warp, and this lane's query.
+struct Walk {
+  float hx, hy, hz;               // half extents of the active queries' box around ref
+  float rm2;                      // squared radius of the walk (box to node, box to particle)
+  float qx, qy, qz, rhof2;        // this lane: query relative to ref, squared radius (< 0: idle)
+  unsigned at;                    // shared address of the lane's next hit
+  unsigned past;                  // hits not kept
+};
+
+__device__ __forceinline__ unsigned shared_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Appends a place or word to the lane's hits when D <= r2; the address moves on for every hit.
+template <bool kStatic>
+__device__ __forceinline__ void append(float D, float r2, unsigned v, unsigned& at) {
+  if (kStatic)
+    asm volatile("{\n .reg .pred p;\n setp.le.f32 p, %1, %2;\n @p st.shared.u16 [%0], %3;\n @p add.u32 %0, %0, 68;\n}"
+                 : "+r"(at) : "f"(D), "f"(r2), "r"(v) : "memory");
+  else
+    asm volatile("{\n .reg .pred p;\n setp.le.f32 p, %1, %2;\n @p st.shared.u32 [%0], %3;\n @p add.u32 %0, %0, 132;\n}"
+                 : "+r"(at) : "f"(D), "f"(r2), "r"(v) : "memory");
+}
+
+// 32 candidates of the queue from b on against every lane's ball.  A hit is appended at once,
+// under a predicate: static, its place; otherwise a word of the upper bits of D and the place.
+// (Hits kept as bits and visited afterwards took 8000 instructions per leaf of 500 candidates
+// against 4500: a leaf's candidates are near one another, so a few lanes have most of the hits
+// among 32 of them and the others wait.)
+// Past full the lane's hits are only counted (static: its walk ends): the buffers have kSlack
+// rows more than they may keep, and the address is held back every kSlack candidates.
+template <bool kStatic>
+__device__ __forceinline__ void test32(const Queue* Q, int b, Walk& W, unsigned full) {
+  constexpr unsigned kStep = kStatic ? 68 : 4 * kPad;
+  const unsigned long long nx = pack2(-W.qx, -W.qx), ny = pack2(-W.qy, -W.qy), nz = pack2(-W.qz, -W.qz);
+  auto hit = [&](float D, unsigned place) {
+    append<kStatic>(D, W.rhof2, kStatic ? place : (__float_as_uint(D) & ~kPlaceMask) | place, W.at);
+  };
+#pragma unroll 1
+  for (int k = b; k < b + 32; k += 8) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) p[u] = r0 + u < cb ? __ldg(A.pos32 + r0 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int h = k; h < k + 8; h += 4) {
+      const uint4 P = *reinterpret_cast<const uint4*>(Q->place + h);
+      const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(Q->x + h);
+      const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(Q->y + h);
+      const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(Q->z + h);
+      float d0, d1, d2, d3;
+      unsigned long long dx = add2(X.x, nx), dy = add2(Y.x, ny), dz = add2(Z.x, nz);
+      unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), d0, d1);
+      dx = add2(X.y, nx); dy = add2(Y.y, ny); dz = add2(Z.y, nz);
+      unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), d2, d3);
+      hit(d0, P.x);
+      hit(d1, P.y);
+      hit(d2, P.z);
+      hit(d3, P.w);
+    }
+    if (W.at > full) {
+      if (kStatic) W.rhof2 = -1.0f;
+      else W.past += (W.at - full) / kStep;
+      W.at = kStatic ? full + kStep : full;
+    }
+  }
+}
+
+// The leaves whose box comes within the walk's radius of the queries' box (g: lo and hi, in
+// units), for one shift (code), added to tab: level by level, four nodes' children loaded
+// together, since every load waits several hundred cycles.  Returns the new count, or -1 when a
+// level does not fit.
+__device__ __forceinline__ int find_leaves(const KnnArgs& A, const TreeDev& T, const float (&g)[6], float rm2,
+                                           int code, int* tab, int cnt, int* front, int lane) {
+  auto near = [&](int l, int first) -> bool {
+    const int c = first + lane;
+    if (first < 0 || c >= T.lev_n[l]) return false;
+    const float4 a = __ldg(A.na + T.lev_off[l] + c);
+    const float2 b = __ldg(A.nb + T.lev_off[l] + c);
+    const float gx = gap(a.x, a.w, g[0], g[3]), gy = gap(a.y, b.x, g[1], g[4]), gz = gap(a.z, b.y, g[2], g[5]);
+    return gx * gx + gy * gy + gz * gz <= rm2;
+  };
+  const unsigned below = (1u << lane) - 1u;
+  const int top = T.nlev - 1;
+  int nf;
+  {
+    const bool h = near(top, 0);
+    const unsigned m = __ballot_sync(kAll, h);
+    nf = __popc(m);
+    if (top == 0) {
+      if (cnt + nf > kSlots) return -1;
+      if (h) tab[cnt + __popc(m & below)] = lane | code;
+      return cnt + nf;
+    }
+    if (h) front[__popc(m & below)] = lane;
+  }
+#pragma unroll 1
+  for (int l = top - 1; l >= 0; --l) {
+    __syncwarp();
+    const int* from = front + ((top - 1 - l) & 1) * kFront;
+    int* to = l == 0 ? tab : front + ((top - l) & 1) * kFront;
+    const int room = l == 0 ? kSlots : kFront;
+    int n = l == 0 ? cnt : 0;
+    const int tag = l == 0 ? code : 0;
+#pragma unroll 1
+    for (int k = 0; k < nf; k += 4) {
+      int f[4];
+      bool h[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + u;
-          if (r >= cb || r == (int)q) continue;
-          const int ixj = __float_as_int(p[u].w) & (kRow1 ? 0x7FFFFFFF : 2047);
-          const float dx = (p[u].x - Q.fx) + (float)(ixj + xoff) * G.cs[0];
-          const float dy = (p[u].y - Q.fy) + dycf;
-          const float dz = (p[u].z - Q.fz) + dzcf;
-          const float D = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          if (D <= rhof2) {
-            if (n_in < CAP) { buf.w(0, n_in) = __float_as_uint(D); buf.w(1, n_in) = (uint32_t)r; }
-            ++n_in;
-          }
-        }
+      for (int u = 0; u < 4; ++u) f[u] = k + u < nf ? from[k + u] * kLeaf : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) h[u] = near(l, f[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const unsigned m = __ballot_sync(kAll, h[u]);
+        const int at = n + __popc(m & below);
+        n += __popc(m);
+        if (h[u] && at < room) to[at] = (f[u] + lane) | tag;
       }
+    }
+    if (n > room) return -1;
+    nf = n;
+  }
+  return nf;
+}
+
+// The leaves of tab: their particles within the walk's radius of the queries' box are queued and
+// tested, four leaves' particles loaded together.
+template <bool kStatic>
+__device__ __forceinline__ void visit(const KnnArgs& A, const TreeDev& T, Queue* Q, const int* tab,
+                                      int cnt, long long r0, int n, const int3 ref, bool per, Walk& W,
+                                      unsigned full, unsigned over, int lane) {
+  const int4* __restrict__ pq = A.posq + r0;
+  constexpr int kLow = (1 << kShiftBit) - 1;
+  int qn = 0;
+#pragma unroll 1
+  for (int s = 0; s < cnt; s += 4) {
+    int4 c[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = s + u < cnt ? tab[s + u] : -1;
+      const int i = (e & kLow) * kLeaf + lane;
+      c[u] = make_int4(0, 0, 0, -1);
+      if (e >= 0 && i < n) c[u] = __ldg(pq + i);
+      if (per && e >= 0) {
+        const int sc = e >> kShiftBit;
+        c[u].x += (sc % 3 - 1) * T.boxq[0];
+        c[u].y += (sc / 3 - 1) * T.boxq[1];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float x = (float)(c[u].x - ref.x), y = (float)(c[u].y - ref.y), z = (float)(c[u].z - ref.z);
+      const float gx = fmaxf(fabsf(x) - W.hx, 0.f), gy = fmaxf(fabsf(y) - W.hy, 0.f), gz = fmaxf(fabsf(z) - W.hz, 0.f);
+      const bool keep = c[u].w >= 0 && gx * gx + gy * gy + gz * gz <= W.rm2;
+      const unsigned m = __ballot_sync(kAll, keep);
+      const int at = keep ? qn + __popc(m & ((1u << lane) - 1u)) : kQueue + lane;
+      Q->x[at] = x;
+      Q->y[at] = y;
+      Q->z[at] = z;
+      Q->place[at] = (unsigned)((s + u) * 32 + lane);
+      qn += __popc(m);
+    }
+    const bool last = s + 4 >= cnt;
+    if (last && (qn & 31)) {
+      // the rest, padded with candidates no ball holds
+      const int to = (qn + 31) & ~31;
+      if (qn + lane < to) { Q->x[qn + lane] = 3e18f; Q->y[qn + lane] = 0.0f; Q->z[qn + lane] = 0.0f; }
+      qn = to;
+    }
+    __syncwarp();
+    int b = 0;
+#pragma unroll 1
+    for (; b + 32 <= qn; b += 32) test32<kStatic>(Q, b, W, full);
+    __syncwarp();
+    if (b) {
+      qn -= b;
+      float x = 0.f, y = 0.f, z = 0.f;
+      unsigned p = 0;
+      if (lane < qn) { x = Q->x[b + lane]; y = Q->y[b + lane]; z = Q->z[b + lane]; p = Q->place[b + lane]; }
+      __syncwarp();
+      if (lane < qn) { Q->x[lane] = x; Q->y[lane] = y; Q->z[lane] = z; Q->place[lane] = p; }
+      // far too many hits: the lane's walk ends
+      if (!kStatic && W.past > over) W.rhof2 = -1.0f;
+      if (!__any_sync(kAll, W.rhof2 >= 0.0f)) return;
+    }
+  }
+}
+
+// Bound of the error of an FP32 distance apart from the relative 10u: a unit per axis from the
+// quantisation (half of one more from the rounded periodic extent) and 2.5u of the relative
+// coordinates, which reach the half extents plus the radius.
+__device__ __forceinline__ float error_bound(bool per, float reach) {
+  return 1.75f * ((per ? 1.6f : 1.1f) + 2.5f * 5.9604645e-8f * (reach * 1.001f + 64.0f));
+}
+
+// Rank of a candidate from its place.
+__device__ __forceinline__ int rank_of_place(const int* tab, int place, int r0) {
+  return r0 + (tab[place >> 5] & ((1 << kShiftBit) - 1)) * kLeaf + (place & 31);
+}
+
+// Static: around the D of the (K-1)-th (dk), keys below lo are certain members and keys above
+// hi none; inside: every particle as near is hit by the ball of radius rho.
+struct Margins {
+  float lo, hi;
+  bool inside;
+};
+__device__ __forceinline__ Margins margins(float dk, float rho, float E) {
+  const float sq = sqrtf(dk);
+  const float hi_tau = (sq * (1.0f + kRel) * 1.000001f + E) * 1.000001f;
+  const float lo_tau = (sq * (1.0f - kRel) * 0.999999f - E) * 0.999999f;
+  const float tlo = fmaxf((lo_tau - E) / (1.0f + kRel), 0.0f), thi = (hi_tau + E) / (1.0f - kRel);
+  return Margins{tlo * tlo * 0.999999f, thi * thi * 1.000001f, hi_tau <= rho};
+}
+
+// The L-th smallest of a lane's n distinct words.  Counts go like D^(3/2): a threshold with L
+// to L + 3 words is interpolated on D, then the largest four below it are ordered.
+__device__ __forceinline__ uint32_t lth_word(const uint32_t* words, int n, int L, float dmax, int lane) {
+  uint32_t t = 0xFFFFFFFFu;
+  int c = n;
+  if (n - L > 3) {
+    uint32_t lo = 0u, hi = 0xFFFFFFFFu;       // counts clo and chi of the words below them
+    int clo = 0, chi = n;
+    float l3 = 0.0f, h3 = dmax * sqrtf(dmax); // their D^(3/2)
+#pragma unroll 1
+    for (int it = 0; it < 40 && chi - L > 3; ++it) {
+      const float f = ((float)L + 1.5f - (float)clo) / (float)(chi - clo);
+      float g = cbrtf(l3 + f * (h3 - l3));
+      g = g * g;
+      uint32_t x = __float_as_uint(g);
+      if (it >= 8 || x <= lo || x >= hi) x = lo + (hi - lo) / 2u;
+      int k = 0;
+      for (int e = 0; e < n; ++e) k += words[e * kPad + lane] < x ? 1 : 0;
+      const float fx = __uint_as_float(min(x, 0x7F000000u));
+      if (k >= L) { hi = x; chi = k; h3 = fx * sqrtf(fx); } else { lo = x; clo = k; l3 = fx * sqrtf(fx); }
+    }
+    t = hi;
+    c = chi;
+  }
+  uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+  for (int e = 0; e < n; ++e) {
+    uint32_t v = words[e * kPad + lane];
+    if (v >= t) v = 0;
+    uint32_t u = max(m0, v); v = min(m0, v); m0 = u;
+    u = max(m1, v); v = min(m1, v); m1 = u;
+    u = max(m2, v); v = min(m2, v); m2 = u;
+    m3 = max(m3, v);
+  }
+  const int left = c - L;
+  return left == 0 ? m0 : left == 1 ? m1 : left == 2 ? m2 : m3;
+}
+
+// Members of one query from its n words (L <= n <= CAP, its own among them), compacted to the
+// front as ranks; d2max the (K-1)-th d^2.  A word's D lies between its upper bits and the next
+// value of them; with the FP32 error bound that gives the band of words that FP64 decides.
+// 1: done, 0: undecided, -1: the ball must grow.
+__device__ __forceinline__ int members(const KnnArgs& A, const TreeDev& T, uint32_t* words, const int* tab,
+                                       int r0, int self, int n, int L, float rho, float E,
+                                       float rhof2, double x, double y, double z, double& d2max, int lane) {
+  constexpr uint32_t low = kPlaceMask;
+  // the query itself is the smallest: L + 1 words from the bottom
+  const uint32_t wl = lth_word(words, n, L + 1, rhof2, lane);
+  const float hi = sqrtf(__uint_as_float(wl | low)) * (1.0f + 2.0f * kRel) + E;      // of the L-th distance
+  const float lo = sqrtf(__uint_as_float(wl & ~low)) * (1.0f - 2.0f * kRel) - E;
+  if (!(hi * 1.000001f <= rho)) return -1;
+  const float a = fmaxf((lo - E) * (1.0f - 2.0f * kRel), 0.0f), b = (hi + E) * (1.0f + 2.0f * kRel);
+  const uint32_t Tlo = __float_as_uint(a * a * 0.999999f), Thi = __float_as_uint(b * b * 1.000001f);
+  int p_lo = 0, nb = 0;
+  int br[kBand];
+#pragma unroll 2
+  for (int e = 0; e < n; ++e) {
+    const uint32_t w = words[e * kPad + lane];
+    if ((w & ~low) > Thi) continue;
+    const int r = rank_of_place(tab, (int)(w & low), r0);
+    if (r == self) continue;
+    if ((w | low) < Tlo) {
+      words[(p_lo++) * kPad + lane] = (uint32_t)r;
     } else {
-    for (int r = ca; r < cb; ++r) {
-      if (r == (int)q) continue;
-      {
-        long long jj;
-        const double d2 = d2_fp64(A.pos64, r, Q.x, Q.y, Q.z, bx, by, jj);
-        if (d2 <= rho2) {
-          if (n_in < CAP) {
-            const unsigned long long kb = (unsigned long long)__double_as_longlong(d2);
-            buf.w(0, n_in) = (uint32_t)kb;
-            buf.w(1, n_in) = (uint32_t)(kb >> 32);
-            if (LaneBuf<CAP, kMixed>::NW > 2) buf.w(2, n_in) = (uint32_t)jj;
-          }
-          ++n_in;
-        }
-      }
+      if (nb == kBand) return 0;
+      br[nb++] = r;
     }
-    }
-    cur = nxt;
-    ca = na;
-    cb = nb;
-    has_cur = has_nxt;
   }
-  return n_in;
+  const int want = L - p_lo;
+  if (want < 1 || want > nb) return 0;
+  // exact FP64 keys of the band, the `want` smallest by (d^2, caller index), compared as bit
+  // patterns (non-negative doubles order like them)
+  unsigned long long bd[kBand];
+  long long bj[kBand];
+#pragma unroll 1
+  for (int t = 0; t < nb; ++t)
+    bd[t] = (unsigned long long)__double_as_longlong(d2_fp64(A.pos64, br[t], x, y, z, T.box[0], T.box[1], bj[t]));
+  unsigned long long kmax = 0;
+  int wr = p_lo;
+#pragma unroll 1
+  for (int t = 0; t < nb; ++t) {
+    int rank = 0;
+#pragma unroll 1
+    for (int u = 0; u < nb; ++u)
+      if (bd[u] < bd[t] || (bd[u] == bd[t] && bj[u] < bj[t])) rank++;
+    if (rank < want) {
+      words[(wr++) * kPad + lane] = (uint32_t)br[t];
+      kmax = kmax > bd[t] ? kmax : bd[t];
+    }
+  }
+  d2max = __longlong_as_double((long long)kmax);
+  return 1;
 }
 
-// Search of one query.  On success the buffer holds the members in entries [0, L)
-// (unsorted) -- the mixed form their ranks (word 1), the FP64 form their caller indices
-// (word 0) -- and d2max is the (K-1)-th d^2.  The output gathers the rest itself.
-// Returns false when no acceptable radius was found (mixed: also when the FP32 keys
-// cannot decide the members).
-template <int CAP, bool kMixed, bool kRow1>
-__device__ bool lane_query(const KnnArgs& A, const Grid32& G, const GridDev& Gd, const QueryPos& Q, long long q,
-                           float rho, const LaneBuf<CAP, kMixed>& buf, double& d2max) {
-  const int L = A.K - 1;
-  const float E = Gd.E32;
-  const float rel = 10.0f * 5.9604645e-8f;
-  const double bx = Gd.box[0], by = Gd.box[1];
-  const float diag = sqrtf((float)G.dim[0] * G.dim[0] * G.cs[0] * G.cs[0] +
-                           (float)G.dim[1] * G.dim[1] * G.cs[1] * G.cs[1] +
-                           (float)G.dim[2] * G.dim[2] * G.cs[2] * G.cs[2]);
-  float r_lo = 0.0f, r_hi = 0.0f;    // radii known to hold too few / too many candidates
-  for (int att = 0; att < 64; ++att) {
-    bool amb = false;
-    const int n_in = scan_ball<CAP, kMixed, kRow1>(A, G, Gd, Q, q, rho, buf, amb);
-    if (kMixed && amb) return false;
-    // a radius that held too few or too many is rescaled by the count towards the middle
-    // of the acceptable range [L, CAP] (count ~ rho^3), then bisected once both are known
-    if (n_in < L) {
-      if (rho > 2.0f * diag) return false;
-      r_lo = rho;
-      rho = r_hi > 0.0f ? sqrtf(r_lo * r_hi) : grow(rho, n_in, L, CAP);
-      continue;
-    }
-    if (n_in > CAP) {
-      r_hi = rho;
-      rho = r_lo > 0.0f ? sqrtf(r_lo * r_hi) : rho * fmaxf(cbrtf(0.5f * (float)(L + CAP) / (float)n_in), 0.3f);
-      continue;
-    }
-    const int iL = buf.select(n_in, L);
-    if (!kMixed) {
-      // exact keys: the L smallest are the members
-      d2max = __longlong_as_double((long long)(((unsigned long long)buf.w(1, iL) << 32) | buf.w(0, iL)));
-      for (int e = 0; e < L; ++e) buf.w(0, e) = buf.w(2, e);
-      return true;
-    }
-    // FP32 bounds with relative margins far above their own rounding
-    const float sq = sqrtf(__uint_as_float(buf.w(0, iL)));
-    const float hi_tau = (sq * (1.0f + rel) * 1.000001f + E) * 1.00001f;
-    if (hi_tau > rho) {
-      if (rho > 2.0f * diag) return false;
-      r_lo = 0.0f;
-      r_hi = 0.0f;
-      rho = hi_tau * 1.02f;
-      continue;
-    }
-    const float rf = (rho * (1.0f + 2.0f * rel) + 2.0f * E) * 1.000001f;
-    const float rhof2 = rf * rf * 1.000001f;
-    const float lo_tau = (sq * (1.0f - rel) * 0.999999f - E) * 0.99999f;
-    const float tlo = (lo_tau - E) / (1.0f + rel);
-    const float thi = (hi_tau + E) / (1.0f - rel);
-    const uint32_t Tlo = tlo > 0.0f ? __float_as_uint(tlo * tlo * 0.99999f) : 0u;
-    const uint32_t Thi = __float_as_uint(thi * thi * 1.00001f);
-    if (Thi > __float_as_uint(rhof2)) return false;   // band reaches past the ball
-    // certain members (key < T_lo) compacted to the front; band ranks set aside
-    int p_lo = 0, nb = 0;
-    int br[kBand];
-    for (int e = 0; e < n_in; ++e) {
-      const uint32_t k = buf.w(0, e);
-      if (k < Tlo) {
-        buf.w(1, p_lo++) = buf.w(1, e);
-      } else if (k <= Thi) {
-        if (nb == kBand) return false;
-        br[nb++] = (int)buf.w(1, e);
-      }
-    }
-    const int need = L - p_lo;
-    if (need < 1 || need > nb) return false;
-    // exact FP64 keys of the band, the `need` smallest by (d^2, caller index); the keys
-    // are compared as bit patterns (non-negative doubles order like them), on the integer
-    // units rather than the FP64 pipe
-    unsigned long long bd[kBand];
-    long long bj[kBand];
-    for (int t = 0; t < nb; ++t)
-      bd[t] = (unsigned long long)__double_as_longlong(d2_fp64(A.pos64, br[t], Q.x, Q.y, Q.z, bx, by, bj[t]));
-    unsigned long long kmax = 0;
-    int wr = p_lo;
-    for (int t = 0; t < nb; ++t) {
-      int rank = 0;
-      for (int u = 0; u < nb; ++u)
-        if (bd[u] < bd[t] || (bd[u] == bd[t] && bj[u] < bj[t])) rank++;
-      if (rank < need) {
-        buf.w(1, wr++) = (uint32_t)br[t];
-        kmax = kmax > bd[t] ? kmax : bd[t];
-      }
-    }
-    d2max = __longlong_as_double((long long)kmax);
-    return true;
-  }
-  return false;
-}
-
-// Ascending sort of 32 keys held in registers (bitonic network, fully unrolled).
-__device__ __forceinline__ void bitonic32(uint32_t (&c)[32]) {
+// Ascending sort of N keys held in registers (bitonic network, fully unrolled).
+template <int N>
+__device__ __forceinline__ void bitonic(uint32_t (&c)[N]) {
 #pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
+  for (int k = 2; k <= N; k <<= 1) {
 #pragma unroll
     for (int j = k >> 1; j > 0; j >>= 1) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
+      for (int i = 0; i < N; ++i) {
         const int l = i ^ j;
         if (l > i) {
           const uint32_t a = c[i], b = c[l];
@@ -527,245 +531,705 @@ __device__ __forceinline__ void bitonic32(uint32_t (&c)[32]) {
   }
 }
 
-template <int CAP> struct KnnShape {
-  // warps per block: buffers (2 words mixed, 3 FP64) of up to four warps within about
-  // 100 KB of shared memory per block
-  static constexpr int bytes(bool mixed) { return (mixed ? 2 : 3) * CAP * kPad * 4; }
-  static constexpr int wpb(bool mixed) {
-    return bytes(mixed) * 4 <= 104 * 1024 ? 4 : (bytes(mixed) * 2 <= 104 * 1024 ? 2 : 1);
-  }
+// LMAX: K at most.  Shared memory of a warp: the hits (static: places; otherwise CAP words), the
+// leaf table, and a scratch that holds the queue and the upper levels' nodes during a walk and
+// the sort keys (a word a member; the ranks then) and, for K > 32, their order (bytes) at
+// the output.
+template <int LMAX, int CAP, bool kStatic> struct KnnShape {
+  static constexpr int al(int v) { return (v + 15) / 16 * 16; }
+  static constexpr int cap = kStatic ? LMAX + kExtra : CAP;    // hits kept, the query's own among them
+  static constexpr int hits = al((cap + kSlack) * (kStatic ? 34 * 2 : kPad * 4));
+  static constexpr int queue = al((int)sizeof(Queue));
+  static constexpr bool regs = LMAX <= 32;                     // the sort in registers
+  // the sort keys: behind the members in the words when there is room
+  static constexpr bool behind = !kStatic && CAP >= 2 * (LMAX - 1);
+  static constexpr int keys = behind ? 0 : al(LMAX * kPad * 4);
+  static constexpr int out = regs ? keys : keys + al(LMAX * kPad);
+  static constexpr int walk = queue + 2 * kFront * 4;
+  static constexpr int scratch = walk > out ? walk : out;
+  static constexpr int bytes = hits + scratch + kSlots * 4;
+  static constexpr int wpb = 2 * bytes <= 56 * 1024 ? 2 : 1;   // warps per block
+  // blocks an SM's shared memory takes (1 KB of it per block is the system's), for the registers
+  static constexpr int fit = 227 * 1024 / (wpb * bytes + 1024);
+  static constexpr int blocks = fit < 1 ? 1 : fit * wpb < kMaxWarps ? fit : kMaxWarps / wpb;
 };
 
-// kRow1: a context of 1D radial instances (their one-row grids pack the x cell in all the
-// bits of w; the 1D model cannot share a context with the others).
-template <int CAP, bool kMixed, bool kRow1>
-__global__ void __launch_bounds__(128, CAP <= 40 && kMixed ? 6 : 4) k_knn(KnnArgs A) {
-  extern __shared__ uint32_t smem[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  LaneBuf<CAP, kMixed> buf;
-  buf.b = smem + (size_t)w * LaneBuf<CAP, kMixed>::NW * CAP * kPad + lane;
+template <int LMAX, int CAP, bool kStatic>
+__global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnShape<LMAX, CAP, kStatic>::blocks) k_knn(KnnArgs A) {
+  using Sh = KnnShape<LMAX, CAP, kStatic>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31;
+  unsigned char* mine = smem + (size_t)(threadIdx.x >> 5) * Sh::bytes;
+  unsigned short* ids = reinterpret_cast<unsigned short*>(mine);
+  uint32_t* words = reinterpret_cast<uint32_t*>(mine);
+  unsigned char* scratch = mine + Sh::hits;
+  Queue* Q = reinterpret_cast<Queue*>(scratch);
+  int* front = reinterpret_cast<int*>(scratch + Sh::queue);
+  int* tab = reinterpret_cast<int*>(scratch + Sh::scratch);
   const int L = A.K - 1;
-  const long long total = A.list ? (long long)*A.list_n : A.N;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
-    const long long q = A.list ? (long long)A.list[t] : t;
-    const int b = inst_of(A.off, A.n_inst, q);
-    const GridDev& Gd = A.grid[b];
-    Grid32 G;
+  const int total = A.listed ? (int)*A.leaves_n : A.n_leaves * A.parts;
+  // no block-wide barrier below: the warps of a block go their own ways
+#pragma unroll 1
+  for (int it = blockIdx.x * Sh::wpb + (threadIdx.x >> 5); it < total; it += gridDim.x * Sh::wpb) {
+  const int item = A.listed ? A.leaves[it] : it;
+  const int leaf = item / A.parts;
+  const int b = lev_inst(A.leaf_off, A.n_inst, leaf);
+  const TreeDev& T = A.tree[b];
+  const InstDev& P = A.P[b];
+  const long long r0 = A.off[b];
+  const int n = (int)(A.off[b + 1] - r0);
+  const int own = leaf - A.leaf_off[b];
+  const int il = own * kLeaf + lane;
+  const bool have = il < n;
+  const long long q = r0 + (have ? il : 0);
+  const int4 me = have ? __ldg(A.posq + q) : make_int4(0, 0, 0, -1);
+  // this warp's queries: all of the leaf's, or a half or quarter of them
+  const bool mine_q = have && (A.parts == 1 || lane / (kLeaf / A.parts) == item % A.parts);
+  const bool valid = me.w >= 0;
+  const bool per = T.periodic != 0;
+  const float half = per ? 0.5f * (float)min(T.boxq[0], T.boxq[1]) : 0.0f;
+  bool pend = valid && mine_q && (!A.listed || A.dist[q] < 0.0);
+  // ---- first radius
+  float rho = 0.0f;
+  {
+    const double dp = pend ? A.dprev[me.w] : 0.0;
+    float d = (float)(dp * T.inv_q);
+    const bool known = dp > 0.0 && dp < 1e300 && d < 1e18f;
+    if (!known) d = 0.0f;
+    if (kStatic) {
+      // a hair over the exact distance: the margins of members_static (E is about 2 units and
+      // 1e-6 d) and no more, so that a particle beyond the members is rarely hit
+      rho = d * 1.000008f + 8.0f;
+      if (!known) { rho = 0.0f; pend = false; }
+    } else {
+      // moved: over one step most neighbourhoods keep their members nearly, so the last distance
+      // and a little is tried first (the counts of a decorrelated neighbourhood scatter by a
+      // sixth: half of its queries then walk again, wider)
+      rho = known ? kMovedFac * d : 0.0f;
+      const bool open = pend && !(rho > 4.0f);
+      if (__any_sync(kAll, open)) {
+        // unknown: the distance to the eighth nearest of the leaf's other particles, which
+        // hold about half of the particles so near, scaled by the wanted count
+        float near[8];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) { G.cs[a] = Gd.cs32[a]; G.inv[a] = Gd.inv32[a]; G.dim[a] = Gd.dim[a]; }
-    G.per = Gd.periodic != 0;
-    G.cell_off = Gd.cell_off;
-    QueryPos Q;
-    const float4 f = __ldg(A.pos32 + q);
-    const int pk = __float_as_int(f.w);
-    Q.ix = kRow1 ? pk : pk & 2047;
-    Q.iy = kRow1 ? 0 : (pk >> 11) & 2047;
-    Q.iz = kRow1 ? 0 : (pk >> 22) & 1023;
-    Q.fx = f.x; Q.fy = f.y; Q.fz = f.z;
+        for (int k = 0; k < 8; ++k) near[k] = 3e38f;
+#pragma unroll 1
+        for (int o = 1; o < 32; ++o) {
+          const int src = lane ^ o;
+          const int x = __shfl_sync(kAll, me.x, src), y = __shfl_sync(kAll, me.y, src),
+                    z = __shfl_sync(kAll, me.z, src);
+          const bool there = __shfl_sync(kAll, (int)valid, src) != 0;
+          const float dx = (float)(x - me.x), dy = (float)(y - me.y), dz = (float)(z - me.z);
+          float v = there ? dx * dx + dy * dy + dz * dz : 3e38f;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float m = fminf(near[k], v);
+            v = fmaxf(near[k], v);
+            near[k] = m;
+          }
+        }
+        float d2 = 0.0f;
+        int m = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (near[k] < 3e38f) { d2 = near[k]; m = k + 1; }
+        // (its noise and its dependence on the place in the leaf evened out by the leaf's mean)
+        const float d8 = sqrtf(d2);
+        const int no = __popc(__ballot_sync(kAll, open));
+        const float mean = warp_sumf(open ? d8 : 0.0f) / (float)max(no, 1);
+        const float r = d8 < 2.0f * mean && mean < 2.0f * d8 ? 0.25f * d8 + 0.75f * mean : d8;
+        if (open) rho = fmaxf(r * cbrtf(kLeafShare * (float)(L + CAP) / (float)max(m, 1)), 8.0f);
+      }
+    }
+  }
+  // ---- walks
+  bool done = false, near_tie = false;
+  float r_lo = 0.0f, r_hi = 0.0f;                  // radii known to hold too few / too many
+  double X = 0.0, Y = 0.0, Z = 0.0;
+  if (have) {
     const double2* pp = reinterpret_cast<const double2*>(A.pos64 + q);
     const double2 a0 = __ldg(pp), a1 = __ldg(pp + 1);
-    Q.x = a0.x; Q.y = a0.y; Q.z = a1.x;
-    const int ci = (int)__double_as_longlong(a1.y);   // caller index
-    // radius: the last build's d_i when known, else the neighbourhood's density
-    const double dp = A.dprev[ci];
-    const float csmax = fmaxf(G.cs[0], fmaxf(G.cs[1], G.cs[2]));
-    float rho = (dp > 0.0 && dp < 1e30) ? A.rfac * (float)dp : 0.0f;
-    if (!(rho > 1e-4f * csmax)) rho = rho_start(G, A.cstart, Q, L);
-    double d2max = 0.0;
-    const bool ok = lane_query<CAP, kMixed, kRow1>(A, G, Gd, Q, q, rho, buf, d2max);
-    int* row = A.nbr + q * (long long)A.K;
-    if (ok) {
-      row[0] = (int)q;
-      // Sort keys: the caller index.  In the mixed form, when the caller indices leave
-      // room, it carries the member's buffer entry in its low kEB bits, so that the rank is
-      // read back from shared memory instead of gathered from rank_of (2^22 disk, K = 32:
-      // 5.14 -> 4.94 ms per build; with the 40-entry buffer the gathers had measured
-      // slightly faster).
-      constexpr int kEB = CAP <= 64 ? 6 : CAP <= 128 ? 7 : CAP <= 256 ? 8 : 9;
-      const bool packed = kMixed && A.N <= (1LL << (32 - kEB));
-      auto sort_key = [&](int e) -> uint32_t {
-        if (!kMixed) return buf.w(0, e);
-        const uint32_t c = (uint32_t)__ldg(&A.perm[buf.w(1, e)]);
-        return packed ? (c << kEB) | (uint32_t)e : c;
-      };
-      auto rank_of_key = [&](uint32_t k) -> int {
-        return packed ? (int)buf.w(1, (int)(k & ((1u << kEB) - 1u))) : __ldg(&A.rank_of[k]);
-      };
-      if constexpr (CAP <= 40) {
-        // K <= 32: the members' sort keys ordered in registers
-        uint32_t cs[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) cs[e] = e < L ? sort_key(e) : 0xFFFFFFFFu;
-        bitonic32(cs);
-#pragma unroll
-        for (int e = 0; e < 31; ++e)
-          if (e < L) row[1 + e] = rank_of_key(cs[e]);
-      } else if constexpr (CAP == 64) {
-        // K <= 48: each half of the members' sort keys ordered in registers and put back
-        // in word 0 (word 1 keeps the mixed form's ranks), then the halves merged
+    X = a0.x; Y = a0.y; Z = a1.x;
+  }
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          uint32_t cs[32];
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const int i = 32 * h + e;
-            cs[e] = i < L ? sort_key(i) : 0xFFFFFFFFu;
-          }
-          bitonic32(cs);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) buf.w(0, 32 * h + e) = cs[e];
+  for (int att = 0; att < (kStatic ? 1 : kTries); ++att) {
+    // a ball reaching across half a periodic extent meets a particle and its image: exact redo
+    if (pend && per && rho * 1.0001f + 64.0f >= half) {
+      if (!kStatic && att == 0) rho = 0.98f * half - 128.0f;   // an estimate: try the largest
+      if (rho * 1.0001f + 64.0f >= half || !(rho > 0.0f)) pend = false;
+    }
+    // One walk for all pending queries, or several: a walk visits the particles within the
+    // largest radius of the queries' box, so a leaf that straddles a density gradient (a large
+    // box or radius beside a small one) is split in halves along the curve until the volume so
+    // visited is below kSplit times the smallest ball's.
+    int largest = 32;                                // queries of a walk at most
+#pragma unroll 1
+    for (unsigned todo = __ballot_sync(kAll, pend); todo;) {
+      const int first = __ffs(todo) - 1;
+      bool act;
+      int gx0, gx1, gy0, gy1, gz0, gz1;
+      float rmax;
+      int size = largest;
+#pragma unroll 1
+      for (;; size >>= 1) {
+        act = ((todo >> lane) & 1u) && (lane & -size) == (first & -size);
+        gx0 = __reduce_min_sync(kAll, act ? me.x : INT_MAX);
+        gx1 = __reduce_max_sync(kAll, act ? me.x : INT_MIN);
+        gy0 = __reduce_min_sync(kAll, act ? me.y : INT_MAX);
+        gy1 = __reduce_max_sync(kAll, act ? me.y : INT_MIN);
+        gz0 = __reduce_min_sync(kAll, act ? me.z : INT_MAX);
+        gz1 = __reduce_max_sync(kAll, act ? me.z : INT_MIN);
+        rmax = __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(act ? rho : 0.0f)));
+        const float rmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(act ? rho : 3e38f)));
+        const float vol = (0.5f * (float)(gx1 - gx0) + rmax) * (0.5f * (float)(gy1 - gy0) + rmax) *
+                          (0.5f * (float)(gz1 - gz0) + rmax);
+        if (size == 1 || vol <= kSplit * rmin * rmin * rmin) break;
+      }
+      Walk W;
+      const int3 ref = make_int3(gx0 + (gx1 - gx0) / 2, gy0 + (gy1 - gy0) / 2, gz0 + (gz1 - gz0) / 2);
+      W.hx = __int2float_ru(gx1 - ref.x);            // the larger half
+      W.hy = __int2float_ru(gy1 - ref.y);
+      W.hz = __int2float_ru(gz1 - ref.z);
+      const float E = error_bound(per, fmaxf(W.hx, fmaxf(W.hy, W.hz)) + rmax);
+      const float rf = (rho * (1.0f + 2.0f * kRel) + 2.0f * E) * 1.000001f;
+      const float rw = (rmax * (1.0f + 4.0f * kRel) + 4.0f * E) * 1.00001f;
+      const float rhof2 = rf * rf * 1.000001f;
+      W.rhof2 = act ? rhof2 : -1.0f;
+      W.rm2 = rw * rw * 1.00001f;
+      W.qx = (float)(me.x - ref.x);
+      W.qy = (float)(me.y - ref.y);
+      W.qz = (float)(me.z - ref.z);
+      constexpr unsigned kStep = kStatic ? 68 : 4 * kPad;
+      const unsigned base = kStatic ? shared_addr(ids + lane) : shared_addr(words + lane);
+      W.at = base;
+      W.past = 0;
+      // shifts of the candidates by -1, 0 or 1 periodic extents that can reach the queries
+      int ix0 = 0, ix1 = 0, iy0 = 0, iy1 = 0;
+      if (per) {
+        const int rr = (int)rw + 8;
+        if (gx0 - rr < T.maxq[0] - T.boxq[0]) ix0 = -1;
+        if (gx1 + rr > T.boxq[0]) ix1 = 1;
+        if (gy0 - rr < T.maxq[1] - T.boxq[1]) iy0 = -1;
+        if (gy1 + rr > T.boxq[1]) iy1 = 1;
+      }
+      int cnt = 0;
+#pragma unroll 1
+      for (int iy = iy0; iy <= iy1 && cnt >= 0; ++iy)
+#pragma unroll 1
+        for (int ix = ix0; ix <= ix1 && cnt >= 0; ++ix) {
+          const int sx = ix * T.boxq[0], sy = iy * T.boxq[1];
+          const float g[6] = {__int2float_rd(gx0 - sx), __int2float_rd(gy0 - sy), __int2float_rd(gz0),
+                              __int2float_ru(gx1 - sx), __int2float_ru(gy1 - sy), __int2float_ru(gz1)};
+          __syncwarp();
+          cnt = find_leaves(A, T, g, W.rm2, (iy * 3 + ix + 4) << kShiftBit, tab, cnt, front, lane);
         }
-        const int n1 = L < 32 ? L : 32;
-        int i = 0, j = 32;
-        uint32_t a = buf.w(0, 0), bq = buf.w(0, 32);   // past a half's members: 0xFFFFFFFF
-        for (int k = 0; k < L; ++k) {
-          const bool first = a < bq;
-          const uint32_t key = first ? a : bq;
-          if (first) { ++i; a = i < n1 ? buf.w(0, i) : 0xFFFFFFFFu; }
-          else { ++j; bq = j < L ? buf.w(0, j) : 0xFFFFFFFFu; }
-          if (packed) row[1 + k] = rank_of_key(key);
-          else buf.w(1, k) = key;
+      __syncwarp();
+      if (cnt < 0 && size > 1) { largest = size >> 1; continue; }   // its leaves do not fit: fewer queries
+      todo &= ~__ballot_sync(kAll, act);
+      const bool fits = cnt >= 0;
+      if (fits) {
+        visit<kStatic>(A, T, Q, tab, cnt, r0, n, ref, per, W, base + Sh::cap * kStep, (kOver - 1) * CAP, lane);
+      }
+      const int hits = (int)((W.at - base) / kStep + W.past);
+      __syncwarp();
+      // ---- this walk's queries
+      bool ok = false;
+      double d2max = 0.0;
+      constexpr int kEB = LMAX <= 32 ? 6 : LMAX <= 64 ? 7 : LMAX <= 128 ? 8 : 9;   // hits are below cap
+      const bool packed = A.packed != 0;
+      // a hit's particle, and its D from the quantised coordinates (static)
+      auto rank_at = [&](int e) -> int {
+        return kStatic ? rank_of_place(tab, ids[e * 34 + lane], (int)r0) : (int)words[e * kPad + lane];
+      };
+      auto dist_to = [&](const int4 c) -> float {
+        int dx = c.x - me.x, dy = c.y - me.y;
+        if (per) {                                   // the hit is the nearest image
+          const int bqx = T.boxq[0], bqy = T.boxq[1];
+          if (2 * abs(dx) > bqx) dx -= dx > 0 ? bqx : -bqx;
+          if (2 * abs(dy) > bqy) dy -= dy > 0 ? bqy : -bqy;
         }
-        if (!packed) {
+        const float fx = (float)dx, fy = (float)dy, fz = (float)(c.z - me.z);
+        return fmaf(fz, fz, fmaf(fy, fy, fx * fx));
+      };
+      // sort keys; the code of this part is kept small (loops over shared memory), since what does
+      // not fit the instruction cache costs more than the loads
+      uint32_t* keys = Sh::behind ? words + L * kPad : reinterpret_cast<uint32_t*>(scratch);
+      const int ne = kStatic ? A.K : L;              // entries to sort (static: the query's own too)
+      if (kStatic) {
+        // the members' sort keys and their two largest D, from the particles themselves (the
+        // coordinates and the caller index come in one load)
+        if (act && hits == A.K) {
+          float m0 = -1.0f, m1 = -1.0f;
+          int e0 = 0;
+          auto key_of = [&](int e) -> uint32_t {
+            const int4 c = __ldg(A.posq + rank_at(e));
+            const float D = dist_to(c);
+            m1 = fmaxf(m1, fminf(m0, D));
+            if (D > m0) { m0 = D; e0 = e; }
+            if (c.w == me.w) return 0xFFFFFFFFu;     // the query itself: past the members
+            return packed ? ((uint32_t)c.w << kEB) | (uint32_t)e : (uint32_t)c.w;
+          };
 #pragma unroll 4
-          for (int k = 0; k < L; ++k) row[1 + k] = __ldg(&A.rank_of[buf.w(1, k)]);
-        }
-      } else {
-        // K > 48: runs of 32 members' sort keys ordered in registers and put back in word
-        // 0 (word 1 keeps the mixed form's ranks), then the runs merged
-        constexpr int NR = (CAP + 31) / 32;
-#pragma unroll 1
-        for (int h = 0; h < NR && 32 * h < L; ++h) {
-          uint32_t cs[32];
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const int i = 32 * h + e;
-            cs[e] = i < L ? sort_key(i) : 0xFFFFFFFFu;
+          for (int e = 0; e < A.K; ++e) keys[e * kPad + lane] = key_of(e);
+          const Margins g = margins(m0, rho, E);
+          ok = g.inside && m1 < g.lo;
+          if (ok) {
+            long long j;
+            d2max = d2_fp64(A.pos64, rank_at(e0), X, Y, Z, T.box[0], T.box[1], j);
           }
-          bitonic32(cs);
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (32 * h + e < L) buf.w(0, 32 * h + e) = cs[e];
         }
-        uint32_t hd[NR];      // each run's next key (0xFFFFFFFF when it is used up)
-        int ps[NR];
+        if (act && !ok && hits >= A.K && hits < A.K + kExtra) {
+          // a few hits too many, or the largest too near one another (a query in a few
+          // hundred): the largest in order give the K-1-th, and its band is ranked in FP64
+          float m[kExtra + 1];
 #pragma unroll
-        for (int c = 0; c < NR; ++c) {
-          ps[c] = 32 * c;
-          hd[c] = ps[c] < L ? buf.w(0, ps[c]) : 0xFFFFFFFFu;
-        }
-        for (int k = 0; k < L; ++k) {
-          uint32_t key = hd[0];
-          int bi = 0;
+          for (int k = 0; k <= kExtra; ++k) m[k] = -1.0f;
+#pragma unroll 1
+          for (int e = 0; e < hits; ++e) {
+            float v = dist_to(__ldg(A.posq + rank_at(e)));
 #pragma unroll
-          for (int c = 1; c < NR; ++c)
-            if (hd[c] < key) { key = hd[c]; bi = c; }
+            for (int k = 0; k <= kExtra; ++k) { const float u = fmaxf(m[k], v); v = fminf(m[k], v); m[k] = u; }
+          }
+          float dk = m[0];
 #pragma unroll
-          for (int c = 0; c < NR; ++c) {
-            if (c == bi) {
-              ++ps[c];
-              const int end = 32 * c + 32 < L ? 32 * c + 32 : L;
-              hd[c] = ps[c] < end ? buf.w(0, ps[c]) : 0xFFFFFFFFu;
+          for (int k = 1; k < kExtra; ++k)
+            if (k == hits - A.K) dk = m[k];
+          const Margins g = margins(dk, rho, E);
+          if (g.inside) {
+            int w = 0, nb = 0;                       // certain entries (the query's own too), band
+            int br[kBand];
+            bool over = false;
+#pragma unroll 1
+            for (int e = 0; e < hits; ++e) {
+              const unsigned short place = ids[e * 34 + lane];
+              const float D = dist_to(__ldg(A.posq + rank_of_place(tab, place, (int)r0)));
+              if (D < g.lo) {
+                ids[(w++) * 34 + lane] = place;
+              } else if (D <= g.hi) {
+                if (nb < kBand) br[nb++] = place; else over = true;
+              }
+            }
+            const int want = A.K - w;
+            if (!over && want >= 1 && want <= nb) {
+              unsigned long long bd[kBand], kmax = 0;
+              long long bj[kBand];
+#pragma unroll 1
+              for (int k = 0; k < nb; ++k)
+                bd[k] = (unsigned long long)__double_as_longlong(
+                    d2_fp64(A.pos64, rank_of_place(tab, br[k], (int)r0), X, Y, Z, T.box[0], T.box[1], bj[k]));
+#pragma unroll 1
+              for (int k = 0; k < nb; ++k) {
+                int rank = 0;
+#pragma unroll 1
+                for (int u = 0; u < nb; ++u)
+                  if (bd[u] < bd[k] || (bd[u] == bd[k] && bj[u] < bj[k])) rank++;
+                if (rank < want) {
+                  ids[(w++) * 34 + lane] = (unsigned short)br[k];
+                  kmax = kmax > bd[k] ? kmax : bd[k];
+                }
+              }
+              d2max = __longlong_as_double((long long)kmax);
+              ok = true;
+#pragma unroll 1
+              for (int e = 0; e < A.K; ++e) {
+                const uint32_t c = (uint32_t)__ldg(&A.posq[rank_at(e)].w);
+                keys[e * kPad + lane] = c == (uint32_t)me.w ? 0xFFFFFFFFu : packed ? (c << kEB) | (uint32_t)e : c;
+              }
             }
           }
-          if (packed) row[1 + k] = rank_of_key(key);
-          else buf.w(1, k) = key;
         }
-        if (!packed) {
-#pragma unroll 4
-          for (int k = 0; k < L; ++k) row[1 + k] = __ldg(&A.rank_of[buf.w(1, k)]);
+        if (act && !ok) {
+          pend = false;
+          if (!fits) near_tie = true;
+          // ties within the error bounds go straight to the exact search
+          if (hits >= A.K && hits < A.K + kExtra) near_tie = true;
+        }
+      } else if (act) {
+        if (!fits) {
+          pend = false;                              // the walk's leaves do not fit: exact search
+        } else if (hits <= L) {
+          r_lo = rho;
+          rho = r_hi > 0.0f ? sqrtf(r_lo * r_hi) : grow(rho, hits, L, CAP);
+        } else if (hits > CAP) {
+          r_hi = rho;
+          rho = r_lo > 0.0f ? sqrtf(r_lo * r_hi)
+                            : rho * (hits > kOver * CAP ? 0.5f : cbrtf(0.5f * (float)(L + CAP) / (float)hits));
+        } else {
+          const int got = members(A, T, words, tab, (int)r0, (int)q, hits, L, rho, E, rhof2, X, Y, Z,
+                                            d2max, lane);
+          ok = got > 0;
+          if (got < 0) { r_lo = rho; rho *= 1.05f; r_hi = 0.0f; }
+          if (got == 0) pend = false;
         }
       }
-      const double d = sqrt(d2max);
-      A.dist[q] = d;
-      const double Vq = sample_volume(A.P[b], d, Q.x, Q.y);
-      A.V[q] = Vq;
-      if (A.pref32) A.pref32[q] = (float)rate_prefactor(A.P[b], Vq, A.K, true);
-      A.dprev[ci] = d;
-    } else if (kMixed) {
-      // the FP64 form redoes it
-      const unsigned long long slot = atomicAdd(A.redo_n, 1ull);
-      A.redo[slot] = (int)q;
-      atomicAdd((unsigned long long*)&A.st[A.P[b].unit0].knn_redo, 1ull);
+      if (ok) { pend = false; done = true; }
+      const unsigned okm = __ballot_sync(kAll, ok);
+      if (okm) {
+        // the members in ascending caller index: sort keys are the caller index with, when the
+        // indices leave room, the member's entry in the low bits
+        auto sort_key = [&](int e) -> uint32_t {
+          const uint32_t c = (uint32_t)__ldg(&A.posq[rank_at(e)].w);
+          return packed ? (c << kEB) | (uint32_t)e : c;
+        };
+        auto rank_of_key = [&](uint32_t k) -> int {
+          return packed ? rank_at((int)(k & ((1u << kEB) - 1u))) : __ldg(&A.rank_of[k]);
+        };
+        int* rows = A.nbr + (r0 + (long long)own * kLeaf) * A.K;      // the leaf's first row
+        if constexpr (Sh::regs) {
+          // Sorted in registers; the ranks then go through shared memory and out row by row: a
+          // row is one 128-byte store for K = 32, where each lane storing its own row touched
+          // 32 sectors per element.
+          uint32_t* out = keys;
+          if (ok) {
+            if (!kStatic) {
+#pragma unroll 4
+              for (int e = 0; e < L; ++e) keys[e * kPad + lane] = sort_key(e);
+            }
+            uint32_t cs[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) cs[e] = e < ne ? keys[e * kPad + lane] : 0xFFFFFFFFu;
+            bitonic<32>(cs);
+#pragma unroll
+            for (int e = 0; e < 32 - 1; ++e)
+              if (e < L) keys[e * kPad + lane] = cs[e];
+#pragma unroll 4
+            for (int e = 0; e < L; ++e) out[e * kPad + lane] = (uint32_t)rank_of_key(keys[e * kPad + lane]);
+          }
+          __syncwarp();
+#pragma unroll 1
+          for (unsigned m = okm; m; m &= m - 1u) {
+            const int l = __ffs(m) - 1;
+            int* row = rows + l * A.K;
+            for (int k = lane; k < A.K; k += 32)
+              row[k] = k == 0 ? (int)(r0 + own * kLeaf + l) : (int)out[(k - 1) * kPad + l];
+          }
+          __syncwarp();
+        } else {
+          // runs of 32 sort keys ordered in registers, then merged: the order of the entries
+          // (packed) or the caller indices themselves
+          unsigned char* order = scratch + Sh::keys;
+          constexpr int NR = (LMAX + 31) / 32;
+          if (ok) {
+#pragma unroll 1
+            for (int h = 0; h < NR && 32 * h < ne; ++h) {
+              uint32_t run[32];
+#pragma unroll
+              for (int e = 0; e < 32; ++e) {
+                const int i = 32 * h + e;
+                run[e] = i < ne ? (kStatic ? keys[i * kPad + lane] : sort_key(i)) : 0xFFFFFFFFu;
+              }
+              bitonic<32>(run);
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (32 * h + e < ne) keys[(32 * h + e) * kPad + lane] = run[e];
+            }
+            uint32_t hd[NR];      // each run's next key (0xFFFFFFFF when it is used up)
+            int ps[NR];
+#pragma unroll
+            for (int c = 0; c < NR; ++c) {
+              ps[c] = 32 * c;
+              hd[c] = ps[c] < ne ? keys[ps[c] * kPad + lane] : 0xFFFFFFFFu;
+            }
+#pragma unroll 1
+            for (int k = 0; k < L; ++k) {
+              uint32_t key = hd[0];
+              int bi = 0;
+#pragma unroll
+              for (int c = 1; c < NR; ++c)
+                if (hd[c] < key) { key = hd[c]; bi = c; }
+#pragma unroll
+              for (int c = 0; c < NR; ++c) {
+                if (c == bi) {
+                  ++ps[c];
+                  const int end = 32 * c + 32 < ne ? 32 * c + 32 : ne;
+                  hd[c] = ps[c] < end ? keys[ps[c] * kPad + lane] : 0xFFFFFFFFu;
+                }
+              }
+              if (packed) order[k * kPad + lane] = (unsigned char)(key & ((1u << kEB) - 1u));
+              else rows[(long long)lane * A.K + 1 + k] = __ldg(&A.rank_of[key]);
+            }
+            if (!packed) rows[(long long)lane * A.K] = (int)q;
+          }
+          __syncwarp();
+          if (packed)
+#pragma unroll 1
+            for (unsigned m = okm; m; m &= m - 1u) {
+              const int l = __ffs(m) - 1;
+              for (int k = lane; k < A.K; k += 32) {
+                int r = (int)(r0 + own * kLeaf + l);
+                if (k > 0) {
+                  const int e = order[(k - 1) * kPad + l];
+                  r = kStatic ? rank_of_place(tab, ids[e * 34 + l], (int)r0) : (int)words[e * kPad + l];
+                }
+                rows[(long long)l * A.K + k] = r;
+              }
+            }
+          __syncwarp();
+        }
+        if (ok) put_result(A, P, q, me.w, d2max, X, Y);
+      }
+    }
+    if (!__any_sync(kAll, pend)) break;
+  }
+  // ---- undecided queries
+  if (kStatic) {
+    // ties and stragglers to the exact search; a leaf with many undecided queries (the caller
+    // moved the particles, or there is no earlier build) to the general kernel
+    bool left = valid && mine_q && !done && !near_tie;
+    const bool few = __popc(__ballot_sync(kAll, left)) * A.parts <= 8;
+    if (near_tie || (left && few)) A.redo[atomicAdd(A.redo_n, 1ull)] = (int)q;
+    left = left && !few;
+    if (left) A.dist[q] = -1.0;
+    if (__any_sync(kAll, left) && lane == 0) A.leaves[atomicAdd(A.leaves_n, 1ull)] = item;
+  } else if (valid && mine_q && !done && (!A.listed || A.dist[q] < 0.0)) {
+    A.redo[atomicAdd(A.redo_n, 1ull)] = (int)q;
+  }
+  if (mine_q && !valid && !A.listed) {
+    // a coordinate that is not finite: the row stays valid (the particle against itself) with
+    // an infinite measure, so the particle gets no rate; the status reports it
+    for (int k = 0; k < A.K; ++k) A.nbr[q * (long long)A.K + k] = (int)q;
+    A.dist[q] = 0.0;
+    A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
+    if (A.pref32) A.pref32[q] = 0.0f;
+    set_status(&A.st[P.unit0], GD_ST_KNN);
+  }
+  }
+}
+
+// ---------------------------------------------------------------- exact queries
+// The list across a warp: entry t * 32 + lane in ascending (key, caller index).
+template <int KPL>
+struct WarpList {
+  unsigned long long k[KPL];      // bits of d^2
+  int j[KPL], r[KPL];             // caller index and rank
+};
+
+// Inserts one entry (the same in every lane) that is smaller than the list's last.
+template <int KPL>
+__device__ __forceinline__ void insert(WarpList<KPL>& S, unsigned long long nk, int nj, int nr, int lane) {
+  int pos = 0;
+#pragma unroll
+  for (int t = 0; t < KPL; ++t) pos += __popc(__ballot_sync(kAll, S.k[t] < nk || (S.k[t] == nk && S.j[t] < nj)));
+#pragma unroll
+  for (int t = KPL - 1; t >= 0; --t) {
+    unsigned long long uk = __shfl_up_sync(kAll, S.k[t], 1);
+    int uj = __shfl_up_sync(kAll, S.j[t], 1), ur = __shfl_up_sync(kAll, S.r[t], 1);
+    const int tp = t > 0 ? t - 1 : 0;
+    const unsigned long long ck = __shfl_sync(kAll, S.k[tp], 31);
+    const int cj = __shfl_sync(kAll, S.j[tp], 31), cr = __shfl_sync(kAll, S.r[tp], 31);
+    if (lane == 0 && t > 0) { uk = ck; uj = cj; ur = cr; }
+    const int at = t * 32 + lane;
+    if (at > pos) { S.k[t] = uk; S.j[t] = uj; S.r[t] = ur; }
+    else if (at == pos) { S.k[t] = nk; S.j[t] = nj; S.r[t] = nr; }
+  }
+}
+
+// Ascending sort of 32 KPL keys, entry t * 32 + lane (bitonic).
+template <int KPL>
+__device__ __forceinline__ void warp_sort(unsigned long long (&v)[KPL], int lane) {
+  for (int k = 2; k <= 32 * KPL; k <<= 1)
+    for (int s = k >> 1; s > 0; s >>= 1) {
+      if (s >= 32) {
+#pragma unroll
+        for (int t = 0; t < KPL; ++t) {
+#pragma unroll
+          for (int u = t + 1; u < KPL; ++u) {
+            if ((t ^ u) != (s >> 5)) continue;
+            const bool up = ((t * 32 + lane) & k) == 0;
+            if (up ? v[t] > v[u] : v[t] < v[u]) { const unsigned long long a = v[t]; v[t] = v[u]; v[u] = a; }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < KPL; ++t) {
+          const unsigned long long o = __shfl_xor_sync(kAll, v[t], s);
+          const bool up = ((t * 32 + lane) & k) == 0, low = (lane & s) == 0;
+          if (low == up ? o < v[t] : o > v[t]) v[t] = o;
+        }
+      }
+    }
+}
+
+template <int KPL>
+__global__ void __launch_bounds__(128) k_knn_exact(KnnArgs A) {
+  __shared__ int stacks[4][2 * kMaxLev];
+  const int lane = threadIdx.x & 31;
+  int* stack = stacks[threadIdx.x >> 5];
+  const int L = A.K - 1;
+  const long long total = (long long)*A.redo_n;
+  const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  for (long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < total; t += nw) {
+    const int q = A.redo[t];
+    const int b = inst_of(A.off, A.n_inst, q);
+    const TreeDev& T = A.tree[b];
+    const InstDev& P = A.P[b];
+    const long long r0 = A.off[b];
+    const int n = (int)(A.off[b + 1] - r0);
+    const int4 me = __ldg(A.posq + q);
+    const Pos64 c = A.pos64[q];
+    const double bx = T.box[0], by = T.box[1];
+    WarpList<KPL> S;
+#pragma unroll
+    for (int u = 0; u < KPL; ++u) { S.k[u] = ~0ull; S.j[u] = INT_MAX; S.r[u] = q; }
+    unsigned long long wk = ~0ull;                 // the (K-1)-th entry so far
+    int wj = INT_MAX;
+    float rm2 = __int_as_float(0x7F800000);
+    auto leaf_in = [&](int leaf) {
+      const int i = leaf * kLeaf + lane;
+      unsigned long long ck = ~0ull;
+      int cj = INT_MAX, cr = -1;
+      if (i < n && r0 + i != q) {
+        const int w = __ldg(&A.posq[r0 + i].w);
+        if (w >= 0) {
+          long long jj;
+          ck = (unsigned long long)__double_as_longlong(d2_fp64(A.pos64, (int)(r0 + i), c.x, c.y, c.z, bx, by, jj));
+          cj = w;
+          cr = (int)(r0 + i);
+        }
+      }
+      unsigned m = __ballot_sync(kAll, ck < wk || (ck == wk && cj < wj));
+      if (!m) return;
+      while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1u;
+        const unsigned long long nk = __shfl_sync(kAll, ck, src);
+        const int nj = __shfl_sync(kAll, cj, src), nr = __shfl_sync(kAll, cr, src);
+        if (!(nk < wk || (nk == wk && nj < wj))) continue;
+        insert<KPL>(S, nk, nj, nr, lane);
+        unsigned long long kv = S.k[0];
+        int jv = S.j[0];
+#pragma unroll
+        for (int u = 1; u < KPL; ++u)
+          if (u == ((L - 1) >> 5)) { kv = S.k[u]; jv = S.j[u]; }
+        wk = __shfl_sync(kAll, kv, (L - 1) & 31);
+        wj = __shfl_sync(kAll, jv, (L - 1) & 31);
+      }
+      if (wk != ~0ull) {
+        // in units, with room for the truncation of both positions and the box's rounding
+        const float u = __double2float_ru(sqrt(__longlong_as_double((long long)wk)) * T.inv_q) * 1.00001f + 8.0f;
+        rm2 = u * u * 1.00001f;
+      }
+    };
+    // the leaves around the query on the curve first: they bound the rest
+    const int own = (int)(q - r0) / kLeaf, e = (L + 31) / 64 + 1, last = T.lev_n[0] - 1;
+    const int la = max(0, own - e), lb = min(last, own + e);
+    for (int leaf = la; leaf <= lb; ++leaf) leaf_in(leaf);
+    const float qxl = __int2float_rd(me.x), qxh = __int2float_ru(me.x), qyl = __int2float_rd(me.y),
+                qyh = __int2float_ru(me.y), qzl = __int2float_rd(me.z), qzh = __int2float_ru(me.z);
+    const float pbx = (float)T.boxq[0], pby = (float)T.boxq[1];
+    auto children = [&](int l, int first) -> unsigned {
+      const int k = first + lane;
+      bool hit = false;
+      if (k < T.lev_n[l]) {
+        const float4 a = __ldg(A.na + T.lev_off[l] + k);
+        const float2 d = __ldg(A.nb + T.lev_off[l] + k);
+        float gx = gap(a.x, a.w, qxl, qxh), gy = gap(a.y, d.x, qyl, qyh);
+        const float gz = gap(a.z, d.y, qzl, qzh);
+        if (T.periodic) {
+          gx = fminf(gx, fminf(gap(a.x, a.w, qxl - pbx, qxh - pbx), gap(a.x, a.w, qxl + pbx, qxh + pbx)));
+          gy = fminf(gy, fminf(gap(a.y, d.x, qyl - pby, qyh - pby), gap(a.y, d.x, qyl + pby, qyh + pby)));
+          gx = fmaxf(gx - 256.0f, 0.0f);           // the extents' rounding
+          gy = fmaxf(gy - 256.0f, 0.0f);
+        }
+        hit = gx * gx + gy * gy + gz * gz <= rm2;
+      }
+      return __ballot_sync(kAll, hit);
+    };
+    const int top = T.nlev - 1;
+    int l = top, first = 0;
+    unsigned m = children(l, 0);
+    for (;;) {
+      while (m == 0 && l < top) {
+        ++l;
+        m = (unsigned)stack[2 * l];
+        first = stack[2 * l + 1];
+      }
+      if (m == 0) break;
+      const int k = first + __ffs(m) - 1;
+      m &= m - 1u;
+      if (l == 0) {
+        if (k < la || k > lb) leaf_in(k);
+      } else {
+        __syncwarp();
+        if (lane == 0) { stack[2 * l] = (int)m; stack[2 * l + 1] = first; }
+        __syncwarp();
+        --l;
+        first = k * kLeaf;
+        m = children(l, first);
+      }
+    }
+    int* row = A.nbr + q * (long long)A.K;
+    if (wk != ~0ull) {
+      unsigned long long v[KPL];
+#pragma unroll
+      for (int u = 0; u < KPL; ++u)
+        v[u] = u * 32 + lane < L ? ((unsigned long long)(unsigned)S.j[u] << 32) | (unsigned)S.r[u] : ~0ull;
+      warp_sort<KPL>(v, lane);
+#pragma unroll
+      for (int u = 0; u < KPL; ++u)
+        if (u * 32 + lane < L) row[1 + u * 32 + lane] = (int)(unsigned)v[u];
+      if (lane == 0) {
+        row[0] = q;
+        put_result(A, P, q, me.w, __longlong_as_double((long long)wk), c.x, c.y);
+        if (A.pref32) atomicAdd((unsigned long long*)&A.st[P.unit0].knn_redo, 1ull);
+      }
     } else {
-      // no acceptable radius: keep the row valid (the particle against itself) with an
-      // infinite measure, so the particle gets no rate; the status reports it
-      for (int k = 0; k < A.K; ++k) row[k] = (int)q;
-      A.dist[q] = 0.0;
-      A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
-      if (A.pref32) A.pref32[q] = 0.0f;
-      A.dprev[ci] = 0.0;
-      set_status(&A.st[A.P[b].unit0], GD_ST_KNN);
+      // fewer than K-1 others with finite coordinates: a valid row, an infinite measure
+      for (int k = lane; k < A.K; k += 32) row[k] = q;
+      if (lane == 0) {
+        A.dist[q] = 0.0;
+        A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
+        if (A.pref32) A.pref32[q] = 0.0f;
+        A.dprev[me.w] = 0.0;
+        set_status(&A.st[P.unit0], GD_ST_KNN);
+      }
     }
   }
 }
 
-template <int CAP, bool kMixed, bool kRow1>
-static cudaError_t launch_knn_t(gd_ctx* c, const KnnArgs& A) {
-  constexpr int kWarps = KnnShape<CAP>::wpb(kMixed);
-  const int bs = kWarps * 32;
-  const int smem = kWarps * KnnShape<CAP>::bytes(kMixed);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_knn<CAP, kMixed, kRow1>, bs, smem);
-  if (per_sm < 1) per_sm = 1;
-  long long blocks = (long long)c->num_sms * per_sm;
-  if (!A.list) {
-    const long long want = (A.N + bs - 1) / bs;
-    if (blocks > want) blocks = want;
-  }
-  if (blocks < 1) blocks = 1;
-  k_knn<CAP, kMixed, kRow1><<<(int)blocks, bs, smem, c->stream>>>(A);
+// ---------------------------------------------------------------- launchers
+template <int LMAX, int CAP, bool kStatic>
+static cudaError_t launch_knn_t(gd_ctx* c, KnnArgs& A) {
+  using Sh = KnnShape<LMAX, CAP, kStatic>;
+  constexpr int kEB = LMAX <= 32 ? 6 : LMAX <= 64 ? 7 : LMAX <= 128 ? 8 : 9;
+  A.packed = A.N <= (1LL << (32 - kEB)) ? 1 : 0;
+  // few leaves: their queries over more warps (a warp's time is a long chain of dependent steps;
+  // a quarter of the queries has a smaller box, fewer candidates and shorter loops)
+  A.parts = 1;
+  while (A.parts < 4 && A.n_leaves * A.parts * 2LL <= 32LL * c->num_sms) A.parts *= 2;
+  int blocks = (int)((A.n_leaves * (long long)A.parts + Sh::wpb - 1) / Sh::wpb);
+  if (A.listed) blocks = blocks < 8 * c->num_sms ? blocks : 8 * c->num_sms;
+  k_knn<LMAX, CAP, kStatic><<<blocks, 32 * Sh::wpb, Sh::wpb * Sh::bytes, c->stream>>>(A);
   return cudaGetLastError();
 }
 
-template <int CAP, bool kMixed>
+template <int LMAX, int CAP>
 static cudaError_t prepare_t() {
-  constexpr int kWarps = KnnShape<CAP>::wpb(kMixed);
-  const int smem = kWarps * KnnShape<CAP>::bytes(kMixed);
-  cudaError_t e = cudaFuncSetAttribute(k_knn<CAP, kMixed, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(k_knn<LMAX, CAP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       KnnShape<LMAX, CAP, true>::wpb * KnnShape<LMAX, CAP, true>::bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_knn<CAP, kMixed, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = cudaFuncSetAttribute(k_knn<LMAX, CAP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             KnnShape<LMAX, CAP, false>::wpb * KnnShape<LMAX, CAP, false>::bytes);
   return e;
 }
 
-template <bool kMixed>
-static cudaError_t prepare_cap(int K) {
-  if (K <= 32) return prepare_t<34, kMixed>();
-  if (K <= 48) return prepare_t<64, kMixed>();
-  if (K <= 80) return prepare_t<96, kMixed>();
-  if (K <= 128) return prepare_t<144, kMixed>();
-  return prepare_t<272, kMixed>();
-}
-
-// Shared-memory opt-in of the neighbour kernels this context launches (once, before any
-// launch or graph capture).
+// Shared-memory opt-in of the neighbour kernels this context launches (once, before any launch
+// or graph capture).
 cudaError_t knn_prepare(gd_ctx* c) {
-  cudaError_t e = prepare_cap<false>(c->K);
-  if (e == cudaSuccess && c->precision == GD_MIXED) e = prepare_cap<true>(c->K);
-  // the wider buffer of a build after particles moved (K <= 32)
-  if (e == cudaSuccess && c->K <= 32) e = prepare_cap<false>(48);
-  if (e == cudaSuccess && c->K <= 32 && c->precision == GD_MIXED) e = prepare_cap<true>(48);
-  return e;
+  if (c->K <= 32) return prepare_t<32, 96>();
+  if (c->K <= 48) return prepare_t<48, 104>();
+  if (c->K <= 64) return prepare_t<64, 112>();
+  if (c->K <= 128) return prepare_t<128, 208>();
+  return prepare_t<256, 320>();
 }
 
-template <int CAP, bool kMixed>
-static cudaError_t launch_both(gd_ctx* c, const KnnArgs& A) {
-  return c->any_model_r ? launch_knn_t<CAP, kMixed, true>(c, A) : launch_knn_t<CAP, kMixed, false>(c, A);
-}
-
-template <bool kMixed>
-static cudaError_t launch_cap(gd_ctx* c, const KnnArgs& A, bool wide) {
-  // buffer capacity: the K-1 members plus room for the radius margin.  Static builds start
-  // at 1.001 d_i, so for K <= 32 a 34-entry buffer holds the ball, and its 36 KB per block
-  // with at most 80 registers lets 6 blocks share an SM (a 40-entry buffer allowed 5: 5.53
-  // against 5.18 ms per build of the 2^22 disk); after particles moved, the K-th distance
-  // is uncertain and K <= 32 takes the 64-entry buffer
-  if (c->K <= 32) return wide ? launch_both<64, kMixed>(c, A) : launch_both<34, kMixed>(c, A);
-  if (c->K <= 48) return launch_both<64, kMixed>(c, A);
-  if (c->K <= 80) return launch_both<96, kMixed>(c, A);
-  if (c->K <= 128) return launch_both<144, kMixed>(c, A);
-  return launch_both<272, kMixed>(c, A);
+template <bool kStatic>
+static cudaError_t launch_k(gd_ctx* c, KnnArgs& A) {
+  if (A.K <= 32) return launch_knn_t<32, 96, kStatic>(c, A);
+  if (A.K <= 48) return launch_knn_t<48, 104, kStatic>(c, A);
+  if (A.K <= 64) return launch_knn_t<64, 112, kStatic>(c, A);
+  if (A.K <= 128) return launch_knn_t<128, 208, kStatic>(c, A);
+  return launch_knn_t<256, 320, kStatic>(c, A);
 }
 
 cudaError_t launch_knn(gd_ctx* c) {
@@ -773,13 +1237,15 @@ cudaError_t launch_knn(gd_ctx* c) {
   A.N = c->N;
   A.K = c->K;
   A.n_inst = c->n_inst;
+  A.n_leaves = c->n_leaves;
   A.off = c->d_off;
+  A.leaf_off = c->d_lev;
   A.P = c->d_inst;
-  A.grid = c->d_grid;
-  A.cstart = c->d_cell_start;
+  A.tree = c->d_tree;
+  A.na = c->d_node_a;
+  A.nb = c->d_node_b;
+  A.posq = c->d_posq;
   A.pos64 = c->d_pos64;
-  A.pos32 = c->d_pos32;
-  A.perm = c->d_perm;
   A.rank_of = c->d_rank_of;
   A.nbr = c->d_nbr;
   A.dist = c->d_dist;
@@ -787,33 +1253,32 @@ cudaError_t launch_knn(gd_ctx* c) {
   A.pref32 = c->d_pref32;
   A.dprev = c->d_dprev;
   A.st = c->d_state;
+  A.leaves = c->d_heavy;          // free until the sampler
+  A.leaves_n = c->d_counters + 2;
   A.redo = c->d_redo;
   A.redo_n = c->d_counters + 1;
-  A.list = nullptr;
-  A.list_n = nullptr;
-  // static particles: d_i of the last build is exact, and 1.001 d_i (with the search's own
-  // rounding margins) holds the K-1 others and little else: the scan's overscan shrinks with
-  // the ball (1.02 d_i took 6.11 ms per build of the 2^22 disk, 1.001 d_i 5.59 ms); after a
-  // move the K-th distance scatters around it, so the first radius aims at the middle of the
-  // buffer's range instead
-  const bool wide = c->moved;
-  A.rfac = c->moved ? 1.045f : 1.001f;
+  A.listed = 0;
+  A.parts = 1;
+  A.packed = 0;
+  const bool moved = c->moved;
   c->moved = false;
   time_begin(c, 1);
-  cudaError_t e = cudaSuccess;
-  if (c->precision == GD_MIXED) {
-    e = cudaMemsetAsync(A.redo_n, 0, sizeof(unsigned long long), c->stream);
-    if (e == cudaSuccess) e = launch_cap<true>(c, A, wide);
-    // the queries the FP32 keys could not decide, in the FP64 form
-    KnnArgs B = A;
-    B.list = c->d_redo;
-    B.list_n = A.redo_n;
-    if (e == cudaSuccess) e = launch_cap<false>(c, B, wide);
-    c->launches += 2;
-  } else {
-    e = launch_cap<false>(c, A, wide);
+  cudaError_t e = cudaMemsetAsync(c->d_counters + 1, 0, 2 * sizeof(unsigned long long), c->stream);
+  if (e == cudaSuccess && !moved) {
+    e = launch_k<true>(c, A);
+    A.listed = 1;
     c->launches += 1;
   }
+  if (e == cudaSuccess) e = launch_k<false>(c, A);
+  if (e == cudaSuccess) {
+    const int blocks = c->num_sms * 4, L = A.K - 1;
+    if (L <= 32) k_knn_exact<1><<<blocks, 128, 0, c->stream>>>(A);
+    else if (L <= 64) k_knn_exact<2><<<blocks, 128, 0, c->stream>>>(A);
+    else if (L <= 128) k_knn_exact<4><<<blocks, 128, 0, c->stream>>>(A);
+    else k_knn_exact<8><<<blocks, 128, 0, c->stream>>>(A);
+    e = cudaGetLastError();
+  }
+  c->launches += 2;
   time_end(c);
   return e;
 }

@@ -464,16 +464,18 @@ cudaError_t launch_timestep(gd_ctx* c, const gd_dt_rule& r, double* dti_out, uns
   return cudaGetLastError();
 }
 
-__global__ void k_out_knn(long long N, int K, const int* __restrict__ rank_of, const int* __restrict__ perm,
-                          const int* __restrict__ nbr, const double* __restrict__ dist, int* nbr_out,
-                          double* d_out) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= N * K) return;
-  long long i = t / K;
-  int k = (int)(t - i * K);
-  int r = rank_of[i];
-  if (nbr_out) nbr_out[t] = perm[nbr[(long long)r * K + k]];
-  if (d_out && k == 0) d_out[i] = dist[r];
+// A warp per particle in rank order: its row read and written in one piece each (the flat index
+// with a 64-bit division per element took 67 us for 10^5 rows of 128).
+__global__ void __launch_bounds__(256) k_out_knn(long long N, int K, const int* __restrict__ perm,
+                                                 const int* __restrict__ nbr, const double* __restrict__ dist,
+                                                 int* nbr_out, double* d_out) {
+  const int lane = threadIdx.x & 31;
+  const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= N) return;
+  const long long i = perm[r];
+  if (nbr_out)
+    for (int k = lane; k < K; k += 32) nbr_out[i * K + k] = __ldg(&perm[nbr[r * K + k]]);
+  if (d_out && lane == 0) d_out[i] = dist[r];
 }
 
 __global__ void k_out_lam(long long N, const int* __restrict__ rank_of, const double* __restrict__ lam,
@@ -523,9 +525,8 @@ cudaError_t launch_diffuse(gd_ctx* c, double dt) {
 
 cudaError_t launch_outputs_knn(gd_ctx* c, int* nbr_out, double* d_out) {
   if (!nbr_out && !d_out) return cudaSuccess;
-  long long n = c->N * c->K;
-  k_out_knn<<<(int)((n + 255) / 256), 256, 0, c->stream>>>(c->N, c->K, c->d_rank_of, c->d_perm, c->d_nbr,
-                                                           c->d_dist, nbr_out, d_out);
+  k_out_knn<<<(unsigned)((c->N + 7) / 8), 256, 0, c->stream>>>(c->N, c->K, c->d_perm, c->d_nbr, c->d_dist, nbr_out,
+                                                              d_out);
   c->launches += 1;
   return cudaGetLastError();
 }
