@@ -64,7 +64,7 @@ static cudaError_t dalloc(T** p, size_t n) {
 
 static void free_all(gd_ctx* c) {
   void* ptrs[] = {c->d_off, c->d_tile_off, c->d_inst, c->d_tree, c->d_state, c->d_bins, c->d_stile_off,
-                  c->d_kv[0], c->d_kv[1], c->d_digits, c->d_chunk, c->d_lev, c->d_node_a, c->d_node_b, c->d_perm,
+                  c->d_digits, c->d_chunk, c->d_lev, c->d_node_a, c->d_node_b, c->d_perm,
                   c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64, c->d_snap32, c->d_Mr, c->d_dist, c->d_V,
                   c->d_lam, c->d_nbr, c->d_counters, c->d_sums, c->d_dprev, c->d_redo, c->d_gx,
                   c->d_pref32, c->d_contrib, c->d_MJ, c->d_part, c->d_heavy, c->d_unit_i, c->d_unit_r, c->d_gperm,
@@ -218,7 +218,6 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   ok &= dalloc(&c->d_state, c->U) == cudaSuccess;
   ok &= dalloc(&c->d_bins, c->U) == cudaSuccess;
   ok &= dalloc(&c->d_stile_off, n + 1) == cudaSuccess;
-  for (int k = 0; k < 2; ++k) ok &= dalloc(&c->d_kv[k], N) == cudaSuccess;
   ok &= dalloc(&c->d_digits, 256LL * c->n_stiles) == cudaSuccess;
   ok &= dalloc(&c->d_chunk, (size_t)c->sort_passes * c->n_chunks) == cudaSuccess;
   ok &= dalloc(&c->d_lev, c->h_lev.size()) == cudaSuccess;
@@ -237,7 +236,11 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   ok &= dalloc(&c->d_heavy, N) == cudaSuccess;
   ok &= dalloc(&c->d_V, N) == cudaSuccess;
   ok &= dalloc(&c->d_lam, N) == cudaSuccess;
-  ok &= dalloc(&c->d_nbr, (size_t)N * c->K) == cudaSuccess;
+  // the lists; the sort's pairs live there too (8 B a particle each, spent before the search
+  // writes its rows)
+  ok &= dalloc(&c->d_nbr, (size_t)N * std::max(c->K, 4)) == cudaSuccess;
+  c->d_kv[0] = reinterpret_cast<uint2*>(c->d_nbr);
+  c->d_kv[1] = c->d_kv[0] + N;
   if (c->precision == GD_MIXED) {
     ok &= dalloc(&c->d_gx, N) == cudaSuccess;
     ok &= dalloc(&c->d_pref32, N) == cudaSuccess;

@@ -134,6 +134,11 @@ struct gd_ctx {
   bool lists_valid = false;             // neighbour lists built (gd_collide may reuse them)
   bool moved = true;                    // no previous build, or particles moved since it
 
+  // gd_neighbors_fixed: lists alone, in the caller's order and indices, without state to keep
+  bool lists_only = false;
+  int* fix_nbr = nullptr;               // [N*K]
+  double* fix_d = nullptr;              // [N] or null
+
   // timing
   static constexpr int kSlots = 8;
   double ms[kSlots] = {0};

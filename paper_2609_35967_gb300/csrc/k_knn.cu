@@ -34,7 +34,7 @@
 // with its lanes waiting for one another), 55% of the issue slots, about 510 candidates tested
 // per leaf of 32 queries.  Builds of a 2^22-particle disk, K = 32: static 5.0 -> 3.6 ms, first
 // 36.6 -> 16 ms; after a push 10.8 -> 6.5 ms (2^20: 2.6 -> 1.6); K = 48 after a push 14.7 -> 8.3
-// ms.  The code is kept small on purpose (loops not unrolled, the reduced models' volume out of
+// ms.  gd_neighbors_fixed of 50,001 particles, K = 32: 3.6 -> 1.0 ms.  The code is kept small on purpose (loops not unrolled, the reduced models' volume out of
 // line): unrolled, it missed the instruction cache and the same builds took half again as long.
 #include <climits>
 
@@ -56,7 +56,7 @@ constexpr int kMaxWarps = 20;     // warps an SM holds at most, the registers sh
                                   // (16: 4% slower, 24: 5% slower, both by spills or idle slots)
 constexpr int kTries = 6;
 constexpr float kMovedFac = 1.04f;  // after a push: 1.03 to 1.08 within 5% of one another (2^20 disk)
-constexpr float kLeafShare = 0.18f;  // first radius: see k_knn
+constexpr float kLeafShare = 0.24f;  // first radius: see k_knn
 constexpr int kOver = 4;          // a lane with more than kOver times its buffer's entries ends its walk
 constexpr float kSplit = 40.0f;   // see k_knn
 constexpr float kRel = 10.0f * 5.9604645e-8f;
@@ -85,6 +85,8 @@ struct KnnArgs {
   int listed;                     // 1: only the listed leaves and their undecided queries
   int* redo;                      // queries for k_knn_exact
   unsigned long long* redo_n;
+  int fixed;                      // gd_neighbors_fixed: rows in the caller's order and indices, dist (caller
+                                  // order, or null) the only other result
   int parts;                      // warps a leaf's queries are spread over (1, 2 or 4)
   int packed;                     // caller indices leave room for a buffer entry in a sort key
 };
@@ -158,11 +160,31 @@ __device__ __forceinline__ double d2_fp64(const Pos64* __restrict__ pos64, int r
 __device__ __forceinline__ void put_result(const KnnArgs& A, const InstDev& P, long long q, int ci, double d2max,
                                            double x, double y) {
   const double d = sqrt(d2max);
+  if (A.fixed) {
+    if (A.dist) A.dist[ci] = d;
+    return;
+  }
   A.dist[q] = d;
   const double Vq = sample_volume(P, d, x, y);
   A.V[q] = Vq;
   if (A.pref32) A.pref32[q] = (float)rate_prefactor(P, Vq, A.K, true);
   A.dprev[ci] = d;
+}
+
+// A query without K-1 others (or a place): the row stays valid (the particle against itself) with
+// an infinite measure, so the particle gets no rate, and the status reports it.  (Fixed: -1.)
+__device__ __forceinline__ void no_list(const KnnArgs& A, const InstDev& P, long long q, int ci) {
+  if (A.fixed) {
+    for (int k = 0; k < A.K; ++k) A.nbr[(long long)ci * A.K + k] = -1;
+    if (A.dist) A.dist[ci] = -1.0;
+    return;
+  }
+  for (int k = 0; k < A.K; ++k) A.nbr[q * (long long)A.K + k] = (int)q;
+  A.dist[q] = 0.0;
+  A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
+  if (A.pref32) A.pref32[q] = 0.0f;
+  A.dprev[ci] = 0.0;
+  set_status(&A.st[P.unit0], GD_ST_KNN);
 }
 
 // Squared distance between two intervals' or a point's and a box's nearest points, per axis.
@@ -592,7 +614,7 @@ __global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnSha
   // ---- first radius
   float rho = 0.0f;
   {
-    const double dp = pend ? A.dprev[me.w] : 0.0;
+    const double dp = pend && !A.fixed ? A.dprev[me.w] : 0.0;
     float d = (float)(dp * T.inv_q);
     const bool known = dp > 0.0 && dp < 1e300 && d < 1e18f;
     if (!known) d = 0.0f;
@@ -608,24 +630,29 @@ __global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnSha
       rho = known ? kMovedFac * d : 0.0f;
       const bool open = pend && !(rho > 4.0f);
       if (__any_sync(kAll, open)) {
-        // unknown: the distance to the eighth nearest of the leaf's other particles, which
-        // hold about half of the particles so near, scaled by the wanted count
+        // unknown: the distance to the eighth nearest of the particles of this leaf and the two
+        // beside it on the curve, which hold most of the particles so near, scaled by the
+        // wanted count
         float near[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) near[k] = 3e38f;
 #pragma unroll 1
-        for (int o = 1; o < 32; ++o) {
-          const int src = lane ^ o;
-          const int x = __shfl_sync(kAll, me.x, src), y = __shfl_sync(kAll, me.y, src),
-                    z = __shfl_sync(kAll, me.z, src);
-          const bool there = __shfl_sync(kAll, (int)valid, src) != 0;
-          const float dx = (float)(x - me.x), dy = (float)(y - me.y), dz = (float)(z - me.z);
-          float v = there ? dx * dx + dy * dy + dz * dz : 3e38f;
+        for (int w = -1; w <= 1; ++w) {
+          const int iw = il + w * kLeaf;
+          int4 c = me;
+          if (w != 0) c = iw >= 0 && iw < n ? __ldg(A.posq + r0 + iw) : make_int4(0, 0, 0, -1);
+#pragma unroll 1
+          for (int src = 0; src < 32; ++src) {
+            const int x = __shfl_sync(kAll, c.x, src), y = __shfl_sync(kAll, c.y, src), z = __shfl_sync(kAll, c.z, src);
+            const bool there = __shfl_sync(kAll, c.w, src) >= 0 && !(w == 0 && src == lane);
+            const float dx = (float)(x - me.x), dy = (float)(y - me.y), dz = (float)(z - me.z);
+            float v = there ? dx * dx + dy * dy + dz * dz : 3e38f;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const float m = fminf(near[k], v);
-            v = fmaxf(near[k], v);
-            near[k] = m;
+            for (int k = 0; k < 8; ++k) {
+              const float m = fminf(near[k], v);
+              v = fmaxf(near[k], v);
+              near[k] = m;
+            }
           }
         }
         float d2 = 0.0f;
@@ -893,15 +920,19 @@ __global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnSha
             for (int e = 0; e < 32 - 1; ++e)
               if (e < L) keys[e * kPad + lane] = cs[e];
 #pragma unroll 4
-            for (int e = 0; e < L; ++e) out[e * kPad + lane] = (uint32_t)rank_of_key(keys[e * kPad + lane]);
+            for (int e = 0; e < L; ++e) {
+              const uint32_t k = keys[e * kPad + lane];
+              out[e * kPad + lane] = A.fixed ? (packed ? k >> kEB : k) : (uint32_t)rank_of_key(k);
+            }
           }
           __syncwarp();
 #pragma unroll 1
           for (unsigned m = okm; m; m &= m - 1u) {
             const int l = __ffs(m) - 1;
-            int* row = rows + l * A.K;
-            for (int k = lane; k < A.K; k += 32)
-              row[k] = k == 0 ? (int)(r0 + own * kLeaf + l) : (int)out[(k - 1) * kPad + l];
+            const int wl = __shfl_sync(kAll, me.w, l);
+            int* row = A.fixed ? A.nbr + (long long)wl * A.K : rows + l * A.K;
+            const int first = A.fixed ? wl : (int)(r0 + own * kLeaf + l);
+            for (int k = lane; k < A.K; k += 32) row[k] = k == 0 ? first : (int)out[(k - 1) * kPad + l];
           }
           __syncwarp();
         } else {
@@ -955,13 +986,15 @@ __global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnSha
 #pragma unroll 1
             for (unsigned m = okm; m; m &= m - 1u) {
               const int l = __ffs(m) - 1;
+              const int wl = __shfl_sync(kAll, me.w, l);
+              int* row = A.fixed ? A.nbr + (long long)wl * A.K : rows + (long long)l * A.K;
               for (int k = lane; k < A.K; k += 32) {
                 int r = (int)(r0 + own * kLeaf + l);
                 if (k > 0) {
                   const int e = order[(k - 1) * kPad + l];
                   r = kStatic ? rank_of_place(tab, ids[e * 34 + l], (int)r0) : (int)words[e * kPad + l];
                 }
-                rows[(long long)l * A.K + k] = r;
+                row[k] = A.fixed ? __ldg(&A.posq[r].w) : r;
               }
             }
           __syncwarp();
@@ -985,13 +1018,8 @@ __global__ void __launch_bounds__(32 * KnnShape<LMAX, CAP, kStatic>::wpb, KnnSha
     A.redo[atomicAdd(A.redo_n, 1ull)] = (int)q;
   }
   if (mine_q && !valid && !A.listed) {
-    // a coordinate that is not finite: the row stays valid (the particle against itself) with
-    // an infinite measure, so the particle gets no rate; the status reports it
-    for (int k = 0; k < A.K; ++k) A.nbr[q * (long long)A.K + k] = (int)q;
-    A.dist[q] = 0.0;
-    A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
-    if (A.pref32) A.pref32[q] = 0.0f;
-    set_status(&A.st[P.unit0], GD_ST_KNN);
+    // a coordinate that is not finite
+    no_list(A, P, q, ~me.w);
   }
   }
 }
@@ -1158,8 +1186,8 @@ __global__ void __launch_bounds__(128) k_knn_exact(KnnArgs A) {
         m = children(l, first);
       }
     }
-    int* row = A.nbr + q * (long long)A.K;
     if (wk != ~0ull) {
+      int* row = A.nbr + (A.fixed ? me.w : q) * (long long)A.K;
       unsigned long long v[KPL];
 #pragma unroll
       for (int u = 0; u < KPL; ++u)
@@ -1167,22 +1195,14 @@ __global__ void __launch_bounds__(128) k_knn_exact(KnnArgs A) {
       warp_sort<KPL>(v, lane);
 #pragma unroll
       for (int u = 0; u < KPL; ++u)
-        if (u * 32 + lane < L) row[1 + u * 32 + lane] = (int)(unsigned)v[u];
+        if (u * 32 + lane < L) row[1 + u * 32 + lane] = A.fixed ? (int)(v[u] >> 32) : (int)(unsigned)v[u];
       if (lane == 0) {
-        row[0] = q;
+        row[0] = A.fixed ? me.w : q;
         put_result(A, P, q, me.w, __longlong_as_double((long long)wk), c.x, c.y);
         if (A.pref32) atomicAdd((unsigned long long*)&A.st[P.unit0].knn_redo, 1ull);
       }
-    } else {
-      // fewer than K-1 others with finite coordinates: a valid row, an infinite measure
-      for (int k = lane; k < A.K; k += 32) row[k] = q;
-      if (lane == 0) {
-        A.dist[q] = 0.0;
-        A.V[q] = __longlong_as_double(0x7FF0000000000000ll);
-        if (A.pref32) A.pref32[q] = 0.0f;
-        A.dprev[me.w] = 0.0;
-        set_status(&A.st[P.unit0], GD_ST_KNN);
-      }
+    } else if (lane == 0) {
+      no_list(A, P, q, me.w);
     }
   }
 }
@@ -1247,8 +1267,9 @@ cudaError_t launch_knn(gd_ctx* c) {
   A.posq = c->d_posq;
   A.pos64 = c->d_pos64;
   A.rank_of = c->d_rank_of;
-  A.nbr = c->d_nbr;
-  A.dist = c->d_dist;
+  A.fixed = c->lists_only ? 1 : 0;
+  A.nbr = c->lists_only ? c->fix_nbr : c->d_nbr;
+  A.dist = c->lists_only ? c->fix_d : c->d_dist;
   A.V = c->d_V;
   A.pref32 = c->d_pref32;
   A.dprev = c->d_dprev;

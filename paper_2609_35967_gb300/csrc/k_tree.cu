@@ -533,7 +533,7 @@ __global__ void k_broadcast_snapshot(const unsigned long long* __restrict__ tota
 // gathered, every rank-space array written coalesced, and the leaf's box.  The scatter this
 // replaces (lane = caller index, stores at random ranks in partial sectors) moved 467 B per
 // particle through DRAM for about 160.
-template <bool kMixed>
+template <bool kMixed, bool kLists>
 __global__ void __launch_bounds__(256) k_gather(int n_leaves, int n_inst, const int* __restrict__ leaf_off,
                                                 const long long* __restrict__ off, const InstDev* __restrict__ P,
                                                 const TreeDev* __restrict__ tree, const double* __restrict__ x,
@@ -561,16 +561,18 @@ __global__ void __launch_bounds__(256) k_gather(int n_leaves, int n_inst, const 
     const int i = perm[r];
     double xi, yi, zi;
     model_pos(p.model, x[i], y[i], z[i], xi, yi, zi);
-    const double si = s[i], Mi = M[i];
-    rank_of[i] = (int)r;
     Pos64 q;
     q.x = xi; q.y = yi; q.z = zi; q.j = i;
     pos64[r] = q;
-    put_snapshot<kMixed>(p, r, si, Mi, snap64, snap32, Mr);
-    if (kMixed) {
-      double R, Zg;
-      gas_coords(p, xi, yi, zi, R, Zg);
-      gx[r] = make_float4((float)R, (float)Zg, (float)Mi, __int_as_float(fine_bin(si)));
+    if (!kLists) {                                  // kLists: gd_neighbors_fixed, positions alone
+      const double si = s[i], Mi = M[i];
+      rank_of[i] = (int)r;
+      put_snapshot<kMixed>(p, r, si, Mi, snap64, snap32, Mr);
+      if (kMixed) {
+        double R, Zg;
+        gas_coords(p, xi, yi, zi, R, Zg);
+        gx[r] = make_float4((float)R, (float)Zg, (float)Mi, __int_as_float(fine_bin(si)));
+      }
     }
     fin = isfinite(xi) && isfinite(yi) && isfinite(zi);
     if (fin) { u[0] = to_unit(T, 0, xi); u[1] = to_unit(T, 1, yi); u[2] = to_unit(T, 2, zi); }
@@ -734,14 +736,11 @@ cudaError_t launch_tree(gd_ctx* c) {
   }
   const double* s = partner_sizes(c);
   const int nb = (c->n_leaves + 7) / 8;
-  if (c->precision == GD_MIXED)
-    k_gather<true><<<nb, 256, 0, st>>>(c->n_leaves, c->n_inst, c->d_lev, c->d_off, c->d_inst, c->d_tree, c->x, c->y,
-                                       c->z, s, c->M, c->d_perm, c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64,
-                                       c->d_snap32, c->d_Mr, c->d_gx, c->d_node_a, c->d_node_b, c->d_state);
-  else
-    k_gather<false><<<nb, 256, 0, st>>>(c->n_leaves, c->n_inst, c->d_lev, c->d_off, c->d_inst, c->d_tree, c->x, c->y,
-                                        c->z, s, c->M, c->d_perm, c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64,
-                                        c->d_snap32, c->d_Mr, c->d_gx, c->d_node_a, c->d_node_b, c->d_state);
+  auto* gather = c->lists_only ? k_gather<false, true> : c->precision == GD_MIXED ? k_gather<true, false>
+                                                                                  : k_gather<false, false>;
+  gather<<<nb, 256, 0, st>>>(c->n_leaves, c->n_inst, c->d_lev, c->d_off, c->d_inst, c->d_tree, c->x, c->y, c->z, s,
+                             c->M, c->d_perm, c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64, c->d_snap32, c->d_Mr,
+                             c->d_gx, c->d_node_a, c->d_node_b, c->d_state);
   for (int l = 1; l < c->max_lev; ++l) {
     const int* tab = c->h_lev.data() + (size_t)l * (c->n_inst + 1);
     const int nodes = tab[c->n_inst] - tab[0];
