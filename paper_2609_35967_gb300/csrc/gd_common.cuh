@@ -174,12 +174,13 @@ struct BinsDev {
 };
 
 // Per-block tiles of the per-particle passes: tile t covers [lo, hi) of one instance (at
-// most kTile particles, never straddling an instance).  The tile table is derived from the
+// most `tile` particles, never straddling an instance).  The tile table is derived from the
 // offsets: block t belongs to the instance whose tile range contains t.
-constexpr int kTile = 4096;
+constexpr int kTileMin = 256, kTileMax = 4096;
 struct TileMap {
   const long long* off;
   int n_inst;
+  int tile;
   const long long* tile_off;   // [n_inst + 1] first tile of each instance
 };
 
@@ -191,8 +192,8 @@ __device__ __forceinline__ bool tile_range(const TileMap& tm, int tile, int& b, 
   }
   b = l;
   long long t = tile - tm.tile_off[b];
-  lo = tm.off[b] + t * kTile;
-  hi = min(lo + kTile, tm.off[b + 1]);
+  lo = tm.off[b] + t * tm.tile;
+  hi = min(lo + tm.tile, tm.off[b + 1]);
   return lo < hi;
 }
 

@@ -30,6 +30,7 @@ struct gd_ctx {
   long long* d_off = nullptr;           // [n_inst + 1]
   long long* d_tile_off = nullptr;      // [n_inst + 1] first per-particle tile of each instance
   int n_tiles = 0;
+  int tile = gd::kTileMax;              // particles per tile: see gd_create
   gd::InstDev* d_inst = nullptr;        // [n_inst]
   gd::TreeDev* d_tree = nullptr;        // [n_inst] search trees
   gd::StateDev* d_state = nullptr;      // [n_inst]
@@ -158,6 +159,7 @@ inline TileMap tile_map(const gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_off;
   tm.n_inst = c->n_inst;
+  tm.tile = c->tile;
   tm.tile_off = c->d_tile_off;
   return tm;
 }
@@ -169,6 +171,7 @@ inline TileMap bins_map(const gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_uoff;
   tm.n_inst = c->U;
+  tm.tile = c->tile;
   tm.tile_off = c->d_utile_off;
   return tm;
 }

@@ -453,12 +453,31 @@ __device__ __forceinline__ double waiting_time(uint32_t a, uint32_t b, double la
 // same fine bin (one match group) sum the group's values in ascending lane order, and the
 // group's lowest lane adds the sums to the warp's own accumulators acc[k * kNFine + bin].
 // A warp's batches come in a fixed order, so no sum depends on scheduling (no float atomics).
-// fbin < 0: the lane adds nothing.
+// fbin < 0: the lane adds nothing.  A warp whose lanes all add to one bin sums in a butterfly.
 template <typename Acc, int NV>
 __device__ __forceinline__ void warp_bin_add(Acc* acc, int* cnt, int fbin, const Acc (&v)[NV], int lane) {
   const int key = fbin >= 0 ? fbin : kNFine + lane;
   const unsigned grp = __match_any_sync(FULLM, key);
   const int npop = __popc(grp);
+  // one bin for all that add (equal grains, a narrow distribution): a fixed butterfly
+  const unsigned any = __ballot_sync(FULLM, fbin >= 0);
+  if (any == 0u) return;
+  if (__all_sync(FULLM, fbin < 0 || grp == any)) {
+    Acc s[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      s[k] = fbin >= 0 ? v[k] : (Acc)0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(FULLM, s[k], o);
+    }
+    if (fbin >= 0 && lane == __ffs(any) - 1) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k) acc[k * kNFine + fbin] += s[k];
+      if (cnt) cnt[fbin] += npop;
+    }
+    __syncwarp();
+    return;
+  }
   const int nmax = (int)__reduce_max_sync(FULLM, (unsigned)npop);
   Acc sum[NV];
 #pragma unroll
@@ -834,8 +853,8 @@ __global__ void k_bins_reduce(const long long* __restrict__ tile_off, const doub
 __global__ void k_interval(const InstDev* __restrict__ P, StateDev* st, BinsDev* bins, int n_units,
                            const int* __restrict__ unit_inst, int K, int no_audit, int mixed) {
   __shared__ double cnt[kNFine], sM[kNFine], sA[kNFine], sB[kNFine], sE[kNFine];
-  __shared__ double gM[kNFine], gA[kNFine], gB[kNFine], gE[kNFine];
-  __shared__ int gid[kNFine];
+  __shared__ double gA[kNFine], gB[kNFine], gE[kNFine], tA[kNFine], tB[kNFine];
+  __shared__ int gid[kNFine], s_ng;
   const int b = blockIdx.x;    // the unit
   if (b >= n_units) return;
   const InstDev& p = P[unit_inst ? unit_inst[b] : b];
@@ -848,51 +867,65 @@ __global__ void k_interval(const InstDev* __restrict__ P, StateDev* st, BinsDev*
   BinsDev& Bn = bins[b];
   for (int f = threadIdx.x; f < kNFine; f += blockDim.x) {
     cnt[f] = Bn.cnt[f]; sM[f] = Bn.sM[f]; sA[f] = Bn.sA[f]; sB[f] = Bn.sB[f]; sE[f] = Bn.sE[f];
-    gM[f] = 0.0; gA[f] = 0.0; gB[f] = 0.0; gE[f] = 0.0;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double thr = K > 64 ? K : 64;
-  int ng = 0;
-  double acc = 0.0;
-  for (int f = 0; f < kNFine; ++f) {
-    gid[f] = -1;
-    if (cnt[f] == 0.0) continue;
-    gid[f] = ng;
-    acc += cnt[f];
-    if (acc >= thr) { ng++; acc = 0.0; }
+  // the bins' groups by one thread, each group's sums and limits by a thread of its own (one
+  // thread for all took 61 us with 50 groups, mostly its FP64 quotients)
+  if (threadIdx.x == 0) {
+    const double thr = K > 64 ? K : 64;
+    int ng = 0;
+    double acc = 0.0;
+    for (int f = 0; f < kNFine; ++f) {
+      gid[f] = -1;
+      if (cnt[f] == 0.0) continue;
+      gid[f] = ng;
+      acc += cnt[f];
+      if (acc >= thr) { ng++; acc = 0.0; }
+    }
+    if (acc > 0.0) {
+      if (ng > 0) { for (int f = 0; f < kNFine; ++f) if (gid[f] == ng) gid[f] = ng - 1; }
+      else ng = 1;
+    }
+    s_ng = ng;
   }
-  if (acc > 0.0) {
-    if (ng > 0) { for (int f = 0; f < kNFine; ++f) if (gid[f] == ng) gid[f] = ng - 1; }
-    else ng = 1;
-  }
-  for (int f = 0; f < kNFine; ++f) {
-    const int g = gid[f];
-    if (g < 0) continue;
-    gM[g] += sM[f]; gA[g] += sA[f]; gB[g] += sB[f];
-    gE[g] = fmax(gE[g], sE[f]);
-  }
-  for (int f = 0; f < kNFine; ++f) Bn.gid[f] = gid[f];
-  Bn.ngroups = ng;
+  __syncthreads();
+  const int ng = s_ng;
   const double C = (p.audit && !no_audit) ? S.C : 1.0;
+  for (int g = threadIdx.x; g < kNFine; g += blockDim.x) {
+    Bn.gid[g] = gid[g];
+    double sumM = 0.0, sumA = 0.0, sumB = 0.0, maxE = 0.0, A = 0.0, Bm = 0.0;
+    tA[g] = tB[g] = HUGE_VAL;
+    if (g < ng) {
+      for (int f = 0; f < kNFine; ++f)
+        if (gid[f] == g) { sumM += sM[f]; sumA += sA[f]; sumB += sB[f]; maxE = fmax(maxE, sE[f]); }
+      A = sumA / sumM;
+      Bm = sumB / sumM;
+      if (A > 0.0) tA[g] = p.eps * C / A;
+      if (Bm > 0.0) tB[g] = p.eps * p.eps * C * C / Bm;
+    }
+    gE[g] = maxE;
+    gA[g] = A;
+    gB[g] = Bm;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) Bn.ngroups = ng;
   const double dtc = S.tau > 0.0 ? S.tau : p.dt_coll;
-  if (S.hold && S.remain_ticks <= 0) {
+  const bool used_up = S.hold && S.remain_ticks <= 0;
+  __syncthreads();                                   // read by all before thread 0 moves on
+  if (used_up) {
     // a bounded collision step (gd_collide) that is used up: idle until the next one
-    S.dt_exe = 0.0;
-    S.events = 0;
+    if (threadIdx.x == 0) { S.dt_exe = 0.0; S.events = 0; }
     return;
   }
+  for (int g = threadIdx.x; g < kNFine; g += blockDim.x) { Bn.gA[g] = gA[g]; Bn.gB[g] = gB[g]; }
+  if (threadIdx.x != 0) return;
   if (S.remain_ticks <= 0) S.remain_ticks = 1LL << 60;
   const double remain = ldexp((double)S.remain_ticks, -60) * dtc;
   const double dt_cap = remain < p.dt_fn_max ? remain : p.dt_fn_max;
   double dt_ab = HUGE_VAL, e_bind = 0.0;
-  for (int g = 0; g < kNFine; ++g) { Bn.gA[g] = 0.0; Bn.gB[g] = 0.0; }
   for (int g = 0; g < ng; ++g) {
-    const double A = gA[g] / gM[g], Bm = gB[g] / gM[g];
-    Bn.gA[g] = A;
-    Bn.gB[g] = Bm;
-    if (A > 0.0) { const double t = p.eps * C / A; if (t < dt_ab) { dt_ab = t; e_bind = gE[g]; } }
-    if (Bm > 0.0) { const double t = p.eps * p.eps * C * C / Bm; if (t < dt_ab) { dt_ab = t; e_bind = gE[g]; } }
+    if (tA[g] < dt_ab) { dt_ab = tA[g]; e_bind = gE[g]; }
+    if (tB[g] < dt_ab) { dt_ab = tB[g]; e_bind = gE[g]; }
   }
   const double tie = mixed ? fmax(2e-5, 1.5 * (e_bind + 64.0 * 0x1p-24)) : 1e-10;
   const double dt_req = dt_ab < dt_cap ? dt_ab : dt_cap;
@@ -1892,30 +1925,35 @@ __global__ void k_step_done(const StateDev* st, int n_units, int* flag) {
 // fine bins for the next interval.
 __global__ void k_audit(const InstDev* __restrict__ P, StateDev* st, BinsDev* bins, int n_units,
                         const int* __restrict__ unit_inst, int no_audit, double tie) {
-  __shared__ double sM[kNFine], sJ[kNFine], gM[kNFine], gJ[kNFine];
-  __shared__ int gid[kNFine];
+  __shared__ double sM[kNFine], sJ[kNFine];
+  __shared__ int gid[kNFine], s_exceed, s_near;
   const int b = blockIdx.x;    // the unit
   if (b >= n_units) return;
   const InstDev& p = P[unit_inst ? unit_inst[b] : b];
   BinsDev& Bn = bins[b];
   for (int f = threadIdx.x; f < kNFine; f += blockDim.x) {
     sM[f] = Bn.sM[f]; sJ[f] = Bn.sJ[f]; gid[f] = Bn.gid[f];
-    gM[f] = 0.0; gJ[f] = 0.0;
+  }
+  if (threadIdx.x == 0) s_exceed = s_near = 0;
+  __syncthreads();
+  if (p.audit && !no_audit && st[b].dt_exe > 0.0) {
+    // a thread per controller bin
+    const double thr = 2.0 * p.eps * st[b].C;
+    for (int g = threadIdx.x; g < Bn.ngroups; g += blockDim.x) {
+      double gM = 0.0, gJ = 0.0;
+      for (int f = 0; f < kNFine; ++f)
+        if (gid[f] == g) { gM += sM[f]; gJ += sJ[f]; }
+      const double Rg = gJ / gM;
+      if (fabs(Rg - thr) <= tie * thr) atomicAdd(&s_near, 1);
+      if (Rg > thr) s_exceed = 1;
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0 && st[b].dt_exe > 0.0) {   // an idle (held) interval leaves C alone
     StateDev& S = st[b];
     if (p.audit && !no_audit) {
-      for (int f = 0; f < kNFine; ++f)
-        if (gid[f] >= 0) { gM[gid[f]] += sM[f]; gJ[gid[f]] += sJ[f]; }
-      const double thr = 2.0 * p.eps * S.C;
-      bool exceed = false;
-      for (int g = 0; g < Bn.ngroups; ++g) {
-        const double Rg = gJ[g] / gM[g];
-        if (fabs(Rg - thr) <= tie * thr) S.near_audit++;
-        if (Rg > thr) exceed = true;
-      }
-      S.C = exceed ? fmax(0.25, 0.5 * S.C) : fmin(1.0, 1.25 * S.C);
+      S.near_audit += s_near;
+      S.C = s_exceed ? fmax(0.25, 0.5 * S.C) : fmin(1.0, 1.25 * S.C);
     } else {
       S.C = 1.0;
     }

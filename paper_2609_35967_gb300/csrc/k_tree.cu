@@ -714,6 +714,7 @@ cudaError_t launch_tree(gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_off;
   tm.n_inst = c->n_inst;
+  tm.tile = kSortTile;
   tm.tile_off = c->d_stile_off;
   const int nt = c->n_stiles;
   cudaStream_t st = c->stream;
