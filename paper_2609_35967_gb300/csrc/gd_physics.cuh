@@ -158,6 +158,37 @@ __device__ __forceinline__ T turb_dv2(T sa, T sb, T vg2, T tre, int& regime, T& 
   return vg2 * (one / (one + s1) + one / (one + s2));
 }
 
+// 2^-99 < v < 2^99, from the exponent bits (integer work, not the FP64 pipe).
+__device__ __forceinline__ bool mid_range(double v) {
+  return (unsigned)__double2hiint(v) - 0x39C00000u < 0x46200000u - 0x39C00000u;
+}
+__device__ __forceinline__ bool mid_range(float) { return true; }
+
+// The same over one denominator, V_t^2 = V_g^2 (add + num / den), so that the FP64 form takes one
+// quotient (an FP64 division holds the narrow FP64 pipe for ten instructions).  In the tiny
+// regime (s1 - s2)/(s1 + s2) (s1^2/(s1 + t) - s2^2/(s2 + t)) has the factor s1 - s2 twice, which
+// the form here keeps instead of cancelling.
+template <typename T>
+__device__ __forceinline__ int turb_quotient(T s1, T s2, T t, T& num, T& den, T& add) {
+  const T one = (T)1, d = s1 - s2, sum = s1 + s2;
+  add = (T)0;
+  if (s1 < t) {
+    num = d * d * (s1 * s2 + t * sum);
+    den = sum * ((s1 + t) * (s2 + t));
+    return 0;
+  }
+  if (s1 < one) {
+    const T ya = (T)1.6, y = ya * s1 + s2;
+    add = ((T)2 * ya - one) * s1 - s2;
+    num = (T)2 * (one / (one + ya) * (s1 * s1) * y + s2 * s2 * s2);
+    den = sum * y;
+    return 1;
+  }
+  num = (T)2 + sum;
+  den = (one + s1) * (one + s2);
+  return 2;
+}
+
 template <typename T>
 struct PairOut {
   T c0, c1;       // effective channel rates in units of the per-particle prefactor
@@ -202,7 +233,7 @@ __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T 
   PairOut<T> o;
   const T one = (T)1;
   T psi;
-  if constexpr (sizeof(T) == 8) psi = m_j / q.m; else psi = m_j * q.inv_m;
+  psi = m_j * q.inv_m;
   T ncoll = one;
   T vg = (T)0;      // 1e-4 / psi when grouped
   if (psi <= (T)1e-6) {
@@ -217,26 +248,61 @@ __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T 
   T derr = (T)0;
   if (q.mode == GD_KERNEL_PHYSICAL) {
     T St_j = q.g * s_j;
-    T aj, bj;
-    // one quotient for both (an FP64 division is a long sequence on the narrow FP64 pipe)
-    if constexpr (sizeof(T) == 8) bj = one / (one + St_j * St_j); else bj = __fdividef(one, one + St_j * St_j);
-    aj = St_j * bj;
-    T hj = St_j < (T)0.5 ? St_j : (T)0.5;
-    T dvR = q.e2 * (q.ai - aj);
-    T dvZ = q.zo * (q.hi - hj);
-    T dvP = q.e1 * (q.bi - bj);
-    T vb;
-    // mixed form: x rsqrt(x) for the FP32 roots (x > 0 here: masses and c_s are positive)
-    if constexpr (sizeof(T) == 4) { const float xb = q.cB * (q.inv_m + inv_m_j); vb = xb * rsqrtf(xb); }
-    else vb = sqrt(q.cB * (q.inv_m + inv_m_j));
-    T dvB = q.cs < vb ? q.cs : vb;
+    T aj = (T)0, bj;
+    // FP64 form: one quotient for b_j and the turbulent term, and the differences of a = St b and
+    // b = 1/(1 + St^2) as products with St_i - St_j: exactly zero for equal grains, no cancellation
     int regime;
-    T s1, s2;
-    T t2 = turb_dv2<T>(q.St, St_j, q.Vg2, q.tRe, regime, s1, s2);
+    T s1, s2, t2;
+    T hj = St_j < (T)0.5 ? St_j : (T)0.5;
+    T dvZ = q.zo * (q.hi - hj);
+    T dvR, dvP;
+    if constexpr (sizeof(T) == 8) {
+      s1 = q.St > St_j ? q.St : St_j;
+      s2 = q.St > St_j ? St_j : q.St;
+      const T x = one + St_j * St_j;
+      if (mid_range(s1) && mid_range(s2)) {
+        if (mid_range(q.tRe)) {
+          T num, den, add;
+          regime = turb_quotient<T>(s1, s2, q.tRe, num, den, add);
+          const T r = one / (x * den);
+          bj = r * den;
+          t2 = q.Vg2 * (add + num * (r * x));
+        } else {   // alpha = 0: Re^-1/2 infinite
+          bj = one / x;
+          t2 = turb_dv2<T>(q.St, St_j, q.Vg2, q.tRe, regime, s1, s2);
+        }
+        const T w = (q.St - St_j) * (q.bi * bj);
+        dvR = q.e2 * (w * (one - q.St * St_j));
+        dvP = q.e1 * (w * (q.St + St_j));
+      } else {
+        // products of these could leave the FP64 range (a grain far above the disk: St beyond 1e29)
+        bj = one / x;
+        t2 = turb_dv2<T>(q.St, St_j, q.Vg2, q.tRe, regime, s1, s2);
+        dvR = q.e2 * (__dmul_rn(q.St, q.bi) - __dmul_rn(St_j, bj));
+        dvP = q.e1 * (q.bi - bj);
+      }
+    } else {
+      bj = __fdividef(one, one + St_j * St_j);
+      t2 = turb_dv2<T>(q.St, St_j, q.Vg2, q.tRe, regime, s1, s2);
+      aj = St_j * bj;
+      dvR = q.e2 * (q.ai - aj);
+      dvP = q.e1 * (q.bi - bj);
+    }
+    // mixed form: x rsqrt(x) for the FP32 roots (x > 0 here: masses and c_s are positive); FP64
+    // form: the Brownian term enters dv^2 squared, so its root is not taken
+    T dvB = (T)0, dvB2;
+    if constexpr (sizeof(T) == 4) {
+      const float xb = q.cB * (q.inv_m + inv_m_j), vb = xb * rsqrtf(xb);
+      dvB = q.cs < vb ? q.cs : vb;
+      dvB2 = dvB * dvB;
+    } else {
+      const T xb = q.cB * (q.inv_m + inv_m_j), c2 = q.cs * q.cs;
+      dvB2 = c2 < xb ? c2 : xb;
+    }
     const T dvt2 = t2;     // the squared turbulent term enters dv^2 as it is
     T dv, xd;
     if constexpr (sizeof(T) == 4) { xd = dvR * dvR + dvZ * dvZ + dvP * dvP + dvB * dvB + dvt2; dv = xd * rsqrtf(xd); }
-    else { xd = dvR * dvR + dvZ * dvZ + dvP * dvP + dvB * dvB + dvt2; dv = sqrt(xd); }
+    else { xd = dvR * dvR + dvZ * dvZ + dvP * dvP + dvB2 + dvt2; dv = sqrt(xd); }
     T ss = q.s + s_j;
     rate = Nq_j * (ss * ss * dv);
     outcome = (dv < q.vfrag) ? 0 : ((psi <= (T)0.1) ? 1 : 2);
@@ -330,14 +396,14 @@ template <typename T>
 __device__ __forceinline__ void pair_moments(const PairOut<T>& o, T fj1, T fj2, T& a, T& b) {
   if (o.outcome == 0) {
     T J;
-    if constexpr (sizeof(T) == 8) J = log1p(o.ncoll * o.psi) / 3.0; else J = log1pf(o.ncoll * o.psi) * (1.0f / 3.0f);
+    if constexpr (sizeof(T) == 8) J = log1p(o.ncoll * o.psi) * (1.0 / 3.0); else J = log1pf(o.ncoll * o.psi) * (1.0f / 3.0f);
     a = o.c0 * J;
     b = o.c0 * (J * J);
   } else if (o.outcome == 1) {
     T J0, J1;
     if constexpr (sizeof(T) == 8) {
-      J0 = fabs(log1p(-o.ncoll * o.psi) / 3.0);
-      J1 = fabs(log(o.psi) / 3.0);
+      J0 = fabs(log1p(-o.ncoll * o.psi) * (1.0 / 3.0));
+      J1 = fabs(log(o.psi) * (1.0 / 3.0));
     } else {
       J0 = fabsf(log1pf(-o.ncoll * o.psi) * (1.0f / 3.0f));
       J1 = fabsf(logf(o.psi) * (1.0f / 3.0f));

@@ -234,8 +234,8 @@ __device__ __forceinline__ Query<T> live_query(const Fixed<T>& f, double s, doub
     double St = f.gst * s;
     q.s = s; q.m = m; q.inv_m = 1.0 / m;
     q.St = St;
-    q.ai = St / (1.0 + St * St);
     q.bi = 1.0 / (1.0 + St * St);
+    q.ai = St * q.bi;
     q.hi = St < 0.5 ? St : 0.5;
     q.g = f.gst;
     q.e2 = f.e2; q.e1 = f.e1; q.zo = f.zo;
