@@ -223,7 +223,7 @@ constexpr float kU32 = 5.9604645e-8f;     // unit roundoff of FP32, 2^-24
 // and dv^2 by E2 = 2 (2 sum |dv_k| err_k + err_t + 5u dv^2) (a factor 2 of margin).  The
 // decision dv < v_frag is certified when |dv^2 - v_frag^2| > E2 + 4u v_frag^2; psi = m_j/m_i
 // (relative error <= 6u) against 0.1 and 1e-6 with a margin of 16u; N_coll = floor(1e-4/psi)
-// when 1e-4 m_i/m_j (an IEEE quotient, within 5u) lies more than 10u of itself from an
+// when 1e-4 m_i (1/m_j) (within 5u) lies more than 10u of itself from an
 // integer below 2^23, else the caller forms it from the FP64 masses (group64, regroup64); the
 // regime of St1 against
 // Re^-1/2 and 1 with a margin of 2 (eps + 2u).  The channel rates are then within
@@ -237,9 +237,9 @@ __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T 
   T ncoll = one;
   T vg = (T)0;      // 1e-4 / psi when grouped
   if (psi <= (T)1e-6) {
-    // mixed form: 1e-4 m_i / m_j with an IEEE quotient -- within 5u of the FP64 form's
-    // 1e-4 / psi (the roundings of m_i, m_j, 1e-4, the product and the quotient)
-    if constexpr (sizeof(T) == 4) vg = __fdiv_rn(1e-4f * q.m, m_j); else vg = (T)1e-4 / psi;
+    // mixed form: 1e-4 m_i (1/m_j) -- within 5u of the FP64 form's 1e-4 / psi (the roundings of
+    // m_i, 1/m_j, 1e-4 and the two products)
+    if constexpr (sizeof(T) == 4) vg = (1e-4f * q.m) * inv_m_j; else vg = (T)1e-4 / psi;
     ncoll = floor(vg);
   }
   T rate;
@@ -357,30 +357,29 @@ __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T 
   o.derr = derr;
   o.rate = rate;
   o.group64 = group64;
-  if (outcome == 0) {
-    if constexpr (sizeof(T) == 4) o.c0 = (ncoll == one) ? rate : __fdividef(rate, ncoll);
-    else o.c0 = (ncoll == one) ? rate : rate / ncoll;
-    o.c1 = (T)0;
-  } else if (outcome == 1) {
-    if constexpr (sizeof(T) == 4) o.c0 = (ncoll == one) ? (one - psi) * rate : __fdividef((one - psi) * rate, ncoll);
-    else o.c0 = (ncoll == one) ? (one - psi) * rate : (one - psi) * rate / ncoll;
-    o.c1 = psi * rate;
-  } else {
-    o.c0 = rate;
-    o.c1 = (T)0;
+  // one quotient for both grouped outcomes (a warp's lanes have either); a fragmentation has
+  // psi > 0.1, so N_coll = 1
+  const T t0 = outcome == 1 ? (one - psi) * rate : rate;
+  o.c0 = t0;
+  if (ncoll != one) {
+    if constexpr (sizeof(T) == 4) o.c0 = __fdividef(t0, ncoll); else o.c0 = t0 / ncoll;
   }
+  o.c1 = outcome == 1 ? psi * rate : (T)0;
   return o;
 }
 
-// Mixed form: N_coll of a grouped pair from the FP64 masses m_i and m_j, the channel rates
+// Mixed form: N_coll of a grouped pair from the FP64 mass m_i and 1/m_j, the channel rates
 // recomputed with it in FP32 (N_coll rounded to FP32, half a unit more of error).  The FP64
-// form forms floor(1e-4 / (m_j / m_i)); here one FP64 quotient (1e-4 m_i) / m_j, within 4
-// units of the last place of that value, so the two floors differ only within 4e-16 of an
-// integer.  A count within 1e-10 of an integer boundary stays uncertified, which covers that.
-__device__ __forceinline__ void regroup64(PairOut<float>& o, double m_i, double m_j) {
-  const double vg = (1e-4 * m_i) / m_j;
+// form forms floor(1e-4 / (m_j / m_i)); here (1e-4 m_i) (1/m_j), within 4 units of the last place
+// of that value, so the two floors differ only within 4e-16 of an integer.  A count within 1e-10
+// of an integer boundary (and the FP32 rounding of the distance) stays uncertified, which covers
+// that.  In a chain of a heavy grain nearly every event has a lane here: a product and a
+// distance in FP32, not an FP64 quotient and comparisons.
+__device__ __forceinline__ void regroup64(PairOut<float>& o, double m_i, double inv_m_j) {
+  const double vg = (1e-4 * m_i) * inv_m_j;
   const double n = floor(vg);
-  if (vg - n <= 1e-10 * vg || n + 1.0 - vg <= 1e-10 * vg) o.cert = 0;
+  const float fr = (float)(vg - n), lim = 1.0001e-10f * (float)vg;
+  if (!(fr > lim && 1.0f - fr > lim + 2.f * kU32)) o.cert = 0;
   const float nf = (float)n;
   o.ncoll = nf;
   if (o.outcome == 0) o.c0 = __fdividef(o.rate, nf);
@@ -394,22 +393,19 @@ __device__ __forceinline__ void regroup64(PairOut<float>& o, double m_i, double 
 // fragmentation uses the precomputed <J>, <J^2> of particle i.
 template <typename T>
 __device__ __forceinline__ void pair_moments(const PairOut<T>& o, T fj1, T fj2, T& a, T& b) {
-  if (o.outcome == 0) {
-    T J;
-    if constexpr (sizeof(T) == 8) J = log1p(o.ncoll * o.psi) * (1.0 / 3.0); else J = log1pf(o.ncoll * o.psi) * (1.0f / 3.0f);
-    a = o.c0 * J;
-    b = o.c0 * (J * J);
-  } else if (o.outcome == 1) {
-    T J0, J1;
-    if constexpr (sizeof(T) == 8) {
-      J0 = fabs(log1p(-o.ncoll * o.psi) * (1.0 / 3.0));
-      J1 = fabs(log(o.psi) * (1.0 / 3.0));
-    } else {
-      J0 = fabsf(log1pf(-o.ncoll * o.psi) * (1.0f / 3.0f));
-      J1 = fabsf(logf(o.psi) * (1.0f / 3.0f));
+  if (o.outcome != 2) {
+    // one log1p for both (a warp's lanes have either); for a sticking pair it is positive
+    const T x = o.ncoll * o.psi, y = o.outcome == 0 ? x : -x;
+    T J0;
+    if constexpr (sizeof(T) == 8) J0 = fabs(log1p(y) * (1.0 / 3.0)); else J0 = fabsf(log1pf(y) * (1.0f / 3.0f));
+    a = o.c0 * J0;
+    b = o.c0 * (J0 * J0);
+    if (o.outcome == 1) {
+      T J1;
+      if constexpr (sizeof(T) == 8) J1 = fabs(log(o.psi) * (1.0 / 3.0)); else J1 = fabsf(logf(o.psi) * (1.0f / 3.0f));
+      a += o.c1 * J1;
+      b += o.c1 * (J1 * J1);
     }
-    a = o.c0 * J0 + o.c1 * J1;
-    b = o.c0 * (J0 * J0) + o.c1 * (J1 * J1);
   } else {
     a = o.c0 * fj1;
     b = o.c0 * fj2;

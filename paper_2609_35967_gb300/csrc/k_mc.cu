@@ -232,9 +232,17 @@ __device__ __forceinline__ Query<T> live_query(const Fixed<T>& f, double s, doub
   if constexpr (sizeof(T) == 8) {
     Query<T> q;
     double St = f.gst * s;
-    q.s = s; q.m = m; q.inv_m = 1.0 / m;
+    const double x = 1.0 + St * St;
+    q.s = s; q.m = m;
     q.St = St;
-    q.bi = 1.0 / (1.0 + St * St);
+    if (mid_range(m) && mid_range(x)) {   // one quotient for both
+      const double r = 1.0 / (m * x);
+      q.inv_m = r * x;
+      q.bi = r * m;
+    } else {
+      q.inv_m = 1.0 / m;
+      q.bi = 1.0 / x;
+    }
     q.ai = St * q.bi;
     q.hi = St < 0.5 ? St : 0.5;
     q.g = f.gst;
@@ -360,7 +368,7 @@ __device__ __forceinline__ double channels_of(const McArgs& A, const Query<T>& q
     if (jr[t] >= 0) {
       po[t] = pair_channels<T>(q, pt[t].s, pt[t].m, pt[t].Nq, pt[t].inv_m);
       if constexpr (sizeof(T) == 4) {
-        if (po[t].group64) regroup64(po[t], m64, A.snap64[jr[t]].m);
+        if (po[t].group64) regroup64(po[t], m64, A.snap64[jr[t]].inv_m);
       }
       c0[t] = po[t].c0;
       c1[t] = po[t].c1;
@@ -383,7 +391,7 @@ __device__ __forceinline__ double lane_channels(const McArgs& A, const Query<T>&
 // s^3 = 6 m / (pi rho_o).  The mixed form multiplies by the per-particle constant.
 template <typename T>
 __device__ __forceinline__ double cube_of(const Fixed<T>& f, double m) {
-  if constexpr (sizeof(T) == 8) return 6.0 * m / (kPi * f.rho_s); else return m * f.k6;
+  return m * f.k6;
 }
 
 // This lane's channel rates summed in FP32 (slot order), for the mixed form's FP32 prefix.
@@ -551,7 +559,7 @@ __device__ __forceinline__ bool rate_particle(const McArgs& A, const InstDev& P,
     if (k + 1 < A.K) { jn = __ldg(row + k + 1); pn = load_partner<T>(A, jn); }
     PairOut<T> po = pair_channels<T>(q, pt.s, pt.m, pt.Nq, pt.inv_m);
     if constexpr (sizeof(T) == 4) {
-      if (po.group64) regroup64(po, A.snap64[r].m, A.snap64[jn_cur].m);
+      if (po.group64) regroup64(po, A.snap64[r].m, A.snap64[jn_cur].inv_m);
     }
     if constexpr (sizeof(T) == 8) { tot = __dadd_rn(tot, po.c0); tot = __dadd_rn(tot, po.c1); }
     else { tot += po.c0; tot += po.c1; cert = cert && po.cert; }
@@ -1081,7 +1089,7 @@ __device__ __noinline__ Fp64Pick fp64_event(const McArgs& A, long long rp, int b
 // frozen partner pj (Sect. 2.5.2, Eq. frag); sset = 0: s is left to s_of_m64 (s must be set
 // for a fragmentation).  Shared by the FP64 sampler and the deferred settlement so that both
 // form the same states.
-__device__ __forceinline__ double s_of_m64(double rho_s, double m) { return cbrt(6.0 * m / (kPi * rho_s)); }
+__device__ __forceinline__ double s_of_m64(double k6, double m) { return cbrt(m * k6); }
 
 __device__ __forceinline__ void event64(double rho_s, double s_min, unsigned k0, unsigned k1, const Snap64& pj,
                                         int ch, int outcome, double ncoll, unsigned il, unsigned iv, unsigned e,
@@ -1106,6 +1114,12 @@ __device__ __forceinline__ void event64(double rho_s, double s_min, unsigned k0,
     sset = 1;
   }
 }
+
+// A grouped count from here on does not fit FP32 (nor, further up, the log's integer): the mass
+// change takes it from the FP64 masses again.  (Rounded to FP32 it moved a mass by up to 6e-12
+// an event, 1e-11 over a chain of 5,000.)
+constexpr float kCountF32 = 0x1p24f;
+__device__ __forceinline__ double count64(double m_i, double inv_m_j) { return floor((1e-4 * m_i) * inv_m_j); }
 
 // Heavy particles with fewer logged events than this keep the in-line FP64 replay.
 constexpr int kDeferMin = 32;
@@ -1270,7 +1284,26 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
     bool tunc = false;        // mixed form: that decision is the time sum's against dt_exe
     int e = 0, near_ch = 0, near_u = 0;   // per-lane ties, warp-uniform ties
     unsigned h = 0u;
+    // J = sum |ln s'/s| telescopes over a run of events of one direction (growth by sticking,
+    // loss by erosion): one logarithm where the direction turns.  Mixed form: from the FP64
+    // masses at the run's ends, |ln(1 + (m' - m)/m)|/3 in FP32.
     T J = (T)0;
+    double run = kMixed ? m : s;
+    int dir = 0;
+    auto flush_run = [&](double at) {
+      if (dir != 0) {
+        if constexpr (kMixed) J += fabsf(log1pf(__fdiv_rn((float)(at - run), (float)run))) * (1.0f / 3.0f);
+        else J += fabs(log(at / run));
+      }
+      run = at;
+      dir = 0;
+    };
+    // the draws of events dbase .. dbase + 31, a lane each (the words of U_s and
+    // -ln U_w): they depend on the event's
+    // number alone, so a chain pays one generator and one logarithm in 32 events
+    int dbase = INT_MIN;
+    unsigned dz = 0u, dw = 0u;
+    T dnl = (T)0;
     T c0[S], c1[S];
     int jr[S];
     PairOut<T> po[S];
@@ -1290,40 +1323,43 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
     // rounding
     auto pairs_checked = [&]() {
       int bad = 0;
-      float de = 0.0f, cs = 0.0f;
+      float de = 0.0f;
 #pragma unroll
       for (int t2 = 0; t2 < S; ++t2)
         if (jr[t2] >= 0) {
           bad += po[t2].cert ? 0 : 1;
           if constexpr (kMixed) {
             de = fmaf((float)po[t2].derr, (float)(c0[t2] + c1[t2]), de);
-            cs += (float)(c0[t2] + c1[t2]);
           }
         }
       if constexpr (kMixed) {
         bad64 = __any_sync(FULLM, bad != 0);
+        // over the prefix's total, which the lanes' rates sum to within its rounding (1.0001)
         de = warp_sumf(de);
-        cs = warp_sumf(cs);
-        eta = (cs > 0.0f ? __fdividef(de, cs) * 1.0001f : 0.0f) + (2.f * S + 7.f) * u;
+        eta = (totf > 0.0f ? __fdividef(de, totf) * 1.0001f : 0.0f) + (2.f * S + 7.f) * u;
       } else {
         near_ch += bad;
       }
     };
     // the particle's FP64 diameter (mixed form: formed from the FP64 mass when it lags)
     auto s_exact = [&]() { return (kMixed && s_stale) ? diameter_of<T>(cube_of<T>(f, m)) : s; };
-    pairs_checked();
-    if constexpr (!kMixed) {
-      incl = warp_incl_scan(v, lane);
-      tot = __shfl_sync(FULLM, incl, 31);
-    } else {
-      inclf = warp_incl_scanf(lane_sumf<S>(c0, c1, jr), lane);
-      totf = __shfl_sync(FULLM, inclf, 31);
-    }
+    auto prefix = [&]() {
+      if constexpr (!kMixed) {
+        incl = warp_incl_scan(v, lane);
+        tot = __shfl_sync(FULLM, incl, 31);
+      } else {
+        inclf = warp_incl_scanf(lane_sumf<S>(c0, c1, jr), lane);
+        totf = __shfl_sync(FULLM, inclf, 31);
+      }
+      pairs_checked();
+    };
+    prefix();
     for (;;) {
       if (unc) break;
       // partner channel: the first cumulative rate above U_s lambda*
       int chosen = INT_MAX, j = -1, outcome = 0;
       T ncoll_t = (T)1, psi_t = (T)0;
+      double nc64 = 0.0;   // mixed form: the count where the FP64 choice gave it
       bool from_po = true;
       if constexpr (kMixed) {
         bool ok = false;
@@ -1345,13 +1381,12 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
             cumf += c1[t2];
             if (c1[t2] > 0.0f && sel == INT_MAX && tf < cumf) { sel = 2 * k + 1; blo = b1; bhi = cumf; }
           }
-          chosen = sel;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) chosen = min(chosen, __shfl_xor_sync(FULLM, chosen, o));
-          if (chosen != INT_MAX) {
-            const int own = (chosen >> 1) / S;
-            const bool in = (bhi - tf > mg) && (blo == 0.0f || tf - blo > mg);
-            ok = __shfl_sync(FULLM, in, own);
+          // slots ascend with the lanes: the first lane that found one holds the least
+          const unsigned has = __ballot_sync(FULLM, sel != INT_MAX);
+          const unsigned inm = __ballot_sync(FULLM, (bhi - tf > mg) && (blo == 0.0f || tf - blo > mg));
+          if (has != 0u) {
+            chosen = __shfl_sync(FULLM, sel, __ffs(has) - 1);
+            ok = (inm & has & (0u - has)) != 0u;
           }
         }
         if (!ok) {
@@ -1362,6 +1397,7 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
           j = pk.j;
           outcome = pk.outcome;
           ncoll_t = (T)pk.ncoll;
+          nc64 = pk.ncoll;
           psi_t = (T)pk.psi;
           from_po = false;
         }
@@ -1388,10 +1424,10 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
             if (sel == INT_MAX && target < cum) sel = 2 * k + 1;
           }
         }
-        chosen = sel;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) chosen = min(chosen, __shfl_xor_sync(FULLM, chosen, o));
-        if (chosen == INT_MAX) {
+        const unsigned has = __ballot_sync(FULLM, sel != INT_MAX);
+        if (has != 0u) {
+          chosen = __shfl_sync(FULLM, sel, __ffs(has) - 1);
+        } else {
           int ln = lastnz;
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) ln = max(ln, __shfl_xor_sync(FULLM, ln, o));
@@ -1401,50 +1437,75 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
       }
       if (chosen < 0) break;
       const int ch = chosen & 1;
+      const int slot = chosen >> 1;
+      const int owner = slot / S, tsl = slot % S;
+      T pso = (T)0;
+      Snap64 pj;      // s only where it is used: the debris of an erosion
+      pj.N = 0.0;
+      pj.inv_m = 0.0;
       if (from_po) {
         // partner data and outcome from the owning lane
-        const int slot = chosen >> 1;
-        const int owner = slot / S, tsl = slot % S;
         int jo = jr[0], oc = po[0].outcome;
-        T nco = po[0].ncoll, pso = po[0].psi;
+        T nco = po[0].ncoll;
+        pso = po[0].psi;
 #pragma unroll
         for (int t2 = 1; t2 < S; ++t2)
           if (t2 == tsl) { jo = jr[t2]; oc = po[t2].outcome; nco = po[t2].ncoll; pso = po[t2].psi; }
         j = __shfl_sync(FULLM, jo, owner);
         outcome = __shfl_sync(FULLM, oc, owner);
         ncoll_t = __shfl_sync(FULLM, nco, owner);
-        psi_t = __shfl_sync(FULLM, pso, owner);
       }
       if constexpr (kMixed) {
-        if (e < lcap && lane == 0) A.dlog[lbase + e] = make_int4(chosen, j, outcome, (int)ncoll_t);
+        pj.m = A.snap64[j].m;
+        pj.s = 0.0;
+      } else {
+        double pm = pt[0].m, ps = pt[0].s;
+#pragma unroll
+        for (int t2 = 1; t2 < S; ++t2)
+          if (t2 == tsl) { pm = pt[t2].m; ps = pt[t2].s; }
+        pj.m = __shfl_sync(FULLM, pm, owner);
+        pj.s = __shfl_sync(FULLM, ps, owner);
       }
-      const double ncoll = (double)ncoll_t;
-      const Snap64 pj = A.snap64[j];
+      if constexpr (kMixed) {
+        if (e < lcap && lane == 0)
+          A.dlog[lbase + e] = make_int4(chosen, j, outcome, (int)fminf((float)ncoll_t, 0x1p30f));
+      }
+      double ncoll = (double)ncoll_t;
+      if constexpr (kMixed) {
+        if (!from_po) ncoll = nc64;
+        else if (ncoll_t >= (T)kCountF32) ncoll = count64(m, A.snap64[j].inv_m);
+      }
       double m_new, s_new = s;
-      float Jf = 0.0f;   // mixed form: |ln s'/s| of the event from the pair's FP32 psi
+      const int way = outcome == 0 ? 1 : -1;   // of s; a fragmentation ends the run by itself
+      if (outcome == 2 || way != dir) {
+        flush_run(kMixed ? m : s);
+        if (outcome != 2) dir = way;
+      }
       if constexpr (!kMixed) {
         int sset;
         m_new = m;
         event64(f.rho_s, f.s_min, k0, k1, pj, ch, outcome, ncoll, il, iv, (unsigned)e, s_new, m_new, sset);
-        if (!sset) s_new = s_of_m64(f.rho_s, m_new);
+        if (!sset) s_new = s_of_m64(f.k6, m_new);
       } else if (outcome == 0) {
         // mixed form: the pair rates only need the FP32 diameter; the FP64-accurate one is
         // formed when it is needed (a fragmentation, an FP64 decision, the particle's end)
         m_new = fma(ncoll, pj.m, m);
         sf = cbrtf((float)m_new * k6f);
         s_stale = true;
-        Jf = log1pf((float)ncoll_t * (float)psi_t) * (1.0f / 3.0f);
       } else if (outcome == 1 && ch == 0) {
         m_new = fma(-ncoll, pj.m, m);
         sf = cbrtf((float)m_new * k6f);
         s_stale = true;
-        Jf = fabsf(log1pf(-(float)ncoll_t * (float)psi_t)) * (1.0f / 3.0f);
       } else if (outcome == 1) {
+        // debris: the particle takes its partner's state
+        flush_run(m);
+        if (from_po) psi_t = __shfl_sync(FULLM, pso, owner);
+        J += fabsf(logf((float)psi_t)) * (1.0f / 3.0f);
         m_new = pj.m;
-        s_new = pj.s;
+        s_new = A.snap64[j].s;
         sf = (float)s_new;
         s_stale = false;
-        Jf = fabsf(logf((float)psi_t)) * (1.0f / 3.0f);
+        run = m_new;
       } else {
         // fragmentation (Eq. frag): the size from the draw in FP64 in both forms
         U4 w2 = philox(il, iv, (unsigned)e, 1u, k0, k1);
@@ -1455,29 +1516,29 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
         s_new = xr * xr;
         m_new = f.mk * (s_new * s_new * s_new);
         sf = (float)s_new;
-        Jf = 2.0f * fabsf(logf((float)(xr / bq)));
+        J += 2.0f * fabsf(logf((float)(xr / bq)));
+        run = m_new;
       }
-      if constexpr (!kMixed) J += fabs(log(s_new / s));
-      else J += Jf;
+      if constexpr (!kMixed) {
+        if (outcome == 2) { J += fabs(log(s_new / s)); run = s_new; }
+      }
       s = s_new;
       m = m_new;
       h = h * 31u + (unsigned)(chosen + 1);
       ++e;
       if (e >= A.max_events) { if (lane == 0) set_status(&A.st[up], GD_ST_EVENT_CAP); break; }
-      // the next event's draws depend only on its counter: formed before the pair refresh, so
-      // that their integer work fills the refresh's latencies
-      U4 w = philox(il, iv, (unsigned)e, 0u, k0, k1);
+      if (dbase < 0 || e - dbase >= 32) {
+        dbase = e;
+        const U4 w = philox(il, iv, (unsigned)(e + lane), 0u, k0, k1);
+        dz = w.z;
+        dw = w.w;
+        if constexpr (!kMixed) dnl = -log(u01(w.x, w.y));
+        else dnl = neg_log_u01_f32(w.x, w.y);
+      }
       if constexpr (!kMixed) q = live_query<T>(f, s, m);
       else q = live_query_f(f, sf, (float)m);
       v = channels_of<T, S>(A, q, m, jr, pt, c0, c1, po);
-      pairs_checked();
-      if constexpr (!kMixed) {
-        incl = warp_incl_scan(v, lane);
-        tot = __shfl_sync(FULLM, incl, 31);
-      } else {
-        inclf = warp_incl_scanf(lane_sumf<S>(c0, c1, jr), lane);
-        totf = __shfl_sync(FULLM, inclf, 31);
-      }
+      prefix();
       double lam_now = 0.0;   // FP64 lambda*_i (FP64 form; mixed form at an uncertified state)
       if constexpr (!kMixed) {
         lam_now = f.pref * tot;
@@ -1496,21 +1557,22 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
         unc = true;
         break;
       }
-      uw0 = w.z;
-      uw1 = w.w;
-      if constexpr (!kMixed) u_s = u01(w.z, w.w);
+      uw0 = __shfl_sync(FULLM, dz, e - dbase);
+      uw1 = __shfl_sync(FULLM, dw, e - dbase);
+      const T nl = __shfl_sync(FULLM, dnl, e - dbase);
+      if constexpr (!kMixed) u_s = u01(uw0, uw1);
       double dt2;
       if constexpr (!kMixed) {
-        dt2 = waiting_time<T>(w.x, w.y, lam_now);
+        dt2 = nl / lam_now;
         if (fabs((t + dt2) - dte) < 1e-10 * dte) near_u++;
       } else {
         if (bad64) {
+          const U4 w = philox(il, iv, (unsigned)e, 0u, k0, k1);
           dt2 = waiting_time<double>(w.x, w.y, lam_now);   // exact up to FP64 rounding
         } else {
           // lambda* = pref * totf in FP32 when it is in range (the FP32 wait is formed
           // from it anyway), else in FP64
           const float lf = preff * totf;
-          const float nl = neg_log_u01_f32(w.x, w.y);
           float d2;
           if (lf > 1e-30f && lf < 1e30f) { d2 = __fdividef(nl, lf); dt2 = (double)d2; }
           else { dt2 = (double)nl / (f.pref * (double)totf); d2 = (float)dt2; }
@@ -1528,6 +1590,7 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
       if (t + dt2 > dte) break;
       t = t + dt2;
     }
+    if (!unc) flush_run(kMixed ? m : s);
     if constexpr (kMixed) {
       if (!unc && s_stale) s = diameter_of<T>(cube_of<T>(f, m));
     }
@@ -1650,25 +1713,27 @@ __global__ void __launch_bounds__(32) k_defer_chain(McArgs A) {
   for (int base = 0; base < rec.n; base += 32) {
     const int k = base + lane;
     int4 L = make_int4(0, 0, 0, 0);
-    double pm = 0.0, ps = 0.0;
+    double pm = 0.0, ps = 0.0, pi = 0.0;
     if (k < rec.n) {
       L = A.dlog[rec.lbase + k];
       const Snap64 pj = A.snap64[L.y];
       pm = pj.m;
       ps = pj.s;
+      pi = pj.inv_m;
     }
     const int cnt = min(32, rec.n - base);
     for (int i = 0; i < cnt; ++i) {
       const int ch = __shfl_sync(FULLM, L.x, i) & 1;
       const int oc = __shfl_sync(FULLM, L.z, i);
-      const double nc = (double)__shfl_sync(FULLM, L.w, i);
+      const int lw = __shfl_sync(FULLM, L.w, i);
       Snap64 pj;
       pj.m = __shfl_sync(FULLM, pm, i);
       pj.s = __shfl_sync(FULLM, ps, i);
+      pj.inv_m = __shfl_sync(FULLM, pi, i);
       pj.N = 0.0;
-      pj.inv_m = 0.0;
+      const double nc = lw >= (int)kCountF32 ? count64(m, pj.inv_m) : (double)lw;
       if (oc == 2 && !sset) {   // a fragmentation starts from the FP64 diameter
-        s = s_of_m64(P.rho_s, m);
+        s = s_of_m64(P.k6, m);
         sset = 1;
       }
       event64(P.rho_s, P.s_min, P.key0, P.key1, pj, ch, oc, nc, il, iv, (unsigned)(base + i), s, m, sset);
@@ -1697,7 +1762,7 @@ __global__ void __launch_bounds__(256) k_defer_states(McArgs A) {
     for (int k = blockIdx.x * wpb + (threadIdx.x >> 5); k <= rec.n; k += gridDim.x * wpb) {
       DState* Sk = A.dstate + rec.sbase + k;
       const double m = Sk->m;
-      const double s = Sk->sset ? Sk->s : s_of_m64(P.rho_s, m);
+      const double s = Sk->sset ? Sk->s : s_of_m64(P.k6, m);
       const U4 w = philox(il, iv, (unsigned)k, 0u, P.key0, P.key1);
       const Fp64Pick pk = fp64_event<S>(A, r, b, s, m, w.z, w.w, true, lane);
       double lam = pk.lam;
@@ -1711,7 +1776,7 @@ __global__ void __launch_bounds__(256) k_defer_states(McArgs A) {
         const int4 L = A.dlog[rec.lbase + k];
         bad = L.x != pk.chosen ? 1 : 0;
         const DState& Sn = A.dstate[rec.sbase + k + 1];
-        const double s1 = Sn.sset ? Sn.s : s_of_m64(P.rho_s, Sn.m);
+        const double s1 = Sn.sset ? Sn.s : s_of_m64(P.k6, Sn.m);
         J = fabs(log(s1 / s));
       }
       if (lane == 0) {
@@ -1802,7 +1867,7 @@ __global__ void __launch_bounds__(32) k_defer_finish(McArgs A) {
         if (!past) {
           const DState& x = St[rec.n];
           m = x.m;
-          s = x.sset ? x.s : s_of_m64(P.rho_s, x.m);
+          s = x.sset ? x.s : s_of_m64(P.k6, x.m);
           cj = x.j;
           co = x.outcome;
           cn = x.ncoll;
@@ -1811,7 +1876,7 @@ __global__ void __launch_bounds__(32) k_defer_finish(McArgs A) {
         double s1 = s, m1 = m;
         int ss1 = 1;
         event64(P.rho_s, P.s_min, P.key0, P.key1, A.snap64[cj], ch & 1, co, cn, il, iv, (unsigned)e, s1, m1, ss1);
-        if (!ss1) s1 = s_of_m64(P.rho_s, m1);
+        if (!ss1) s1 = s_of_m64(P.k6, m1);
         J += fabs(log(s1 / s));
         s = s1;
         m = m1;
@@ -1848,7 +1913,7 @@ __global__ void __launch_bounds__(32) k_defer_finish(McArgs A) {
   }
   if (!past) {   // the final diameter: that of the state reached
     const DState& x = St[e];
-    s = x.sset ? x.s : s_of_m64(P.rho_s, x.m);
+    s = x.sset ? x.s : s_of_m64(P.k6, x.m);
   }
   if (lane == 0) {
     const int ci = A.perm[r];
@@ -1867,8 +1932,13 @@ __global__ void __launch_bounds__(32) k_defer_finish(McArgs A) {
   }
 }
 
-template <typename T, int S>
-__global__ void __launch_bounds__(64, sizeof(T) == 8 ? 4 : 7) k_sample(McArgs A) {
+// Bound by the latency of the longest chain: of 2^22 particles of a broad disk one takes 3,408
+// events, and SMs ran out of work after 3.4 ms of 8.4.  An event's draws, logarithms and sums are
+// kept off its serial path (8.4 -> 7.8 ms alone, FP64 form of 1.5 million particles 16.7 -> 12).
+// kBlk blocks of 64 fit an SM: four leave a warp the registers to keep an event's values, six have
+// more warps to hide the chunks' loads.  Which: sample_launch.
+template <typename T, int S, int kBlk>
+__global__ void __launch_bounds__(64, kBlk) k_sample(McArgs A) {
   const int lane = threadIdx.x & 31;
   // spatial groups: the round's ranks only (A.act), 32 to a chunk like the full range
   const long long total = A.act ? (long long)*A.act_n : A.N;
@@ -2084,17 +2154,31 @@ cudaError_t launch_interval(gd_ctx* c) {
   return e;
 }
 
-template <typename T, int S>
-static void sample_launch(gd_ctx* c, const McArgs& A) {
+template <typename T, int S, int kBlk>
+static void sample_blocks(gd_ctx* c, const McArgs& A) {
   // 64-thread blocks: the register budget of this kernel then still fills the SM
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<T, S>, 64, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<T, S, kBlk>, 64, 0);
   if (per_sm < 1) per_sm = 1;
   long long chunks = (A.N + 31) / 32;
   long long blocks = (long long)c->num_sms * per_sm;
   if (blocks > (chunks + 1) / 2) blocks = (chunks + 1) / 2;
   if (blocks < 1) blocks = 1;
-  k_sample<T, S><<<(int)blocks, 64, 0, c->stream>>>(A);
+  k_sample<T, S, kBlk><<<(int)blocks, 64, 0, c->stream>>>(A);
+}
+
+// Up to 2^20 particles a warp has at most some 16 chunks and the longest chain decides: four
+// blocks an SM (2^20 broad, K = 48: 2.83 ms against 3.19 with six; eight groups of 2^18: 1.4x).
+// Above, the chunks weigh more: six (2^22: an interval of three contexts at once 8.42 ms against
+// 8.72 with four).  The FP64 form fits four either way.
+template <typename T, int S>
+static void sample_launch(gd_ctx* c, const McArgs& A) {
+  if constexpr (sizeof(T) == 8) {
+    sample_blocks<T, S, 4>(c, A);
+  } else {
+    if (A.N <= (1LL << 20)) sample_blocks<T, S, 4>(c, A);
+    else sample_blocks<T, S, 6>(c, A);
+  }
 }
 
 // The deferred FP64 settlement after the mixed sampler: 32 blocks of 8 warps per deferred
