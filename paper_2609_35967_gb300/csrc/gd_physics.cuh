@@ -417,39 +417,51 @@ __device__ __forceinline__ void pair_moments(const PairOut<T>& o, T fj1, T fj2, 
 // dtheta = h l_theta / r^2 in the meridional plane (cos a - 1 = -2 sin^2(a/2) and sin a in
 // FP32), then scaled by 1 + h v_r / r.  The first half takes phi, theta (both at the old
 // radius), radius; the second half the mirrored order.
-__device__ __forceinline__ void drift_f(double h, double& X, double& Y, double& Z, double VR, double LT,
-                                        double LP, bool first_half) {
-  auto phi = [&]() {
-    const double R2 = X * X + Y * Y;
-    const float dph = (float)(h * LP) / (float)R2;
-    const float s2 = sinf(0.5f * dph);
-    const double c1 = (double)(-2.0f * s2 * s2), s1 = (double)sinf(dph);
-    const double Xr = X + (c1 * X - s1 * Y), Yr = Y + (c1 * Y + s1 * X);
-    X = Xr;
-    Y = Yr;
-  };
-  auto theta = [&]() {
-    const double R = sqrt(X * X + Y * Y), r2 = R * R + Z * Z;
-    const float dth = (float)(h * LT) / (float)r2;
-    const float t2 = sinf(0.5f * dth);
-    const double ct = (double)(-2.0f * t2 * t2), st = (double)sinf(dth);
-    // theta from +z: R' = R cos + Z sin, Z' = Z cos - R sin
-    const double dR = ct * R + st * Z, dZ = ct * Z - st * R;
-    const double f = 1.0 + dR / R;
-    X *= f;
-    Y *= f;
-    Z += dZ;
-  };
-  auto radius = [&]() {
-    const double r = sqrt(X * X + Y * Y + Z * Z);
-    const double f = 1.0 + h * VR / r;
-    X *= f;
-    Y *= f;
-    Z *= f;
-  };
-  // first half: phi, theta (both at the old radius), radius; second half mirrored
-  if (first_half) { phi(); theta(); radius(); }
-  else { radius(); theta(); phi(); }
+__device__ __forceinline__ void drift_phi(double h, double& X, double& Y, double LP) {
+  const double R2 = X * X + Y * Y;
+  const float dph = (float)(h * LP) / (float)R2;
+  const float s2 = sinf(0.5f * dph);
+  const double c1 = (double)(-2.0f * s2 * s2), s1 = (double)sinf(dph);
+  const double Xr = X + (c1 * X - s1 * Y), Yr = Y + (c1 * Y + s1 * X);
+  X = Xr;
+  Y = Yr;
+}
+
+__device__ __forceinline__ void drift_first(double h, double& X, double& Y, double& Z, double VR, double LT,
+                                            double LP) {
+  drift_phi(h, X, Y, LP);
+  const double R = sqrt(X * X + Y * Y), r2 = R * R + Z * Z;
+  const float dth = (float)(h * LT) / (float)r2;
+  const float t2 = sinf(0.5f * dth);
+  const double ct = (double)(-2.0f * t2 * t2), st = (double)sinf(dth);
+  // theta from +z: R' = R cos + Z sin, Z' = Z cos - R sin
+  const double dR = ct * R + st * Z, dZ = ct * Z - st * R;
+  const double f = 1.0 + dR / R;
+  X *= f;
+  Y *= f;
+  Z += dZ;
+  const double r = sqrt(X * X + Y * Y + Z * Z);
+  const double g = 1.0 + h * VR / r;
+  X *= g;
+  Y *= g;
+  Z *= g;
+}
+
+// The second half from the midpoint's radii (r, R and their inverses, which the kick has): the
+// radial step scales both and leaves Z/R, so no root and no quotient is taken again.
+__device__ __forceinline__ void drift_second(double h, double& X, double& Y, double& Z, double VR, double LT,
+                                             double LP, double r, double ir, double R, double iR) {
+  const double f = 1.0 + h * VR * ir;
+  const double zR = Z * iR, Rs = R * f, rs = r * f;
+  Z *= f;
+  const float dth = (float)(h * LT) / (float)(rs * rs);
+  const float t2 = sinf(0.5f * dth);
+  const double ct = (double)(-2.0f * t2 * t2), st = (double)sinf(dth);
+  const double g = f * (1.0 + (ct + st * zR));
+  X *= g;
+  Y *= g;
+  Z += ct * Z - st * Rs;
+  drift_phi(h, X, Y, LP);
 }
 
 }  // namespace gd

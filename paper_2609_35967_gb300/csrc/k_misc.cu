@@ -73,13 +73,13 @@ __global__ void k_push_f(long long N, int n_inst, const long long* __restrict__ 
   const double dt = dt_in < 0.0 ? st[P[b].unit0].dt_exe : dt_in;
   const double h = 0.5 * dt;
   double X = x[i], Y = y[i], Zc = z[i], VR = vr[i], LT = lth[i], LP = lph[i];
-  drift_f(h, X, Y, Zc, VR, LT, LP, true);
+  drift_first(h, X, Y, Zc, VR, LT, LP);
   // kick at the midpoint
   const double R2 = X * X + Y * Y, R = sqrt(R2), r = sqrt(R2 + Zc * Zc);
-  const double ir = 1.0 / r, sth = R * ir, cth = Zc * ir, ir2 = ir * ir;
+  const double ir = 1.0 / r, iR = 1.0 / R, cth = Zc * ir, ir2 = ir * ir, isth = r * iR;
   // f_r = -GM/r^2 + l_theta^2/r^3 + l_phi^2/(r^3 sin^2 theta), r^3 sin^2 theta = r R^2
-  const double fr = (-p.GM + LT * LT * ir + LP * LP * r / R2) * ir2;
-  const double fth = LP * LP * cth * ir2 / (sth * sth * sth);
+  const double fr = (-p.GM + LT * LT * ir + LP * LP * isth * iR) * ir2;
+  const double fth = LP * LP * cth * ir2 * (isth * isth * isth);
   // the gas disk at the midpoint in FP32 (the forms of the FP32 diffusion coefficients)
   const float Rf = (float)R, Zf = (float)Zc;
   const float Om = sqrtf(p.f_GM / Rf) / Rf;
@@ -93,11 +93,11 @@ __global__ void k_push_f(long long N, int n_inst, const long long* __restrict__ 
   const float gam = Om / (gst * (float)s[i]);
   const float kf = gam > 0.0f ? -expm1f(-(float)dt * gam) / gam : (float)dt;
   const double k = (double)kf, kg = (double)(kf * gam);
-  const double ygph = sqrt(1.0 - 2.0 * (double)eta) * sqrt(p.GM * R);
+  const double ygph = sqrt((1.0 - 2.0 * (double)eta) * (p.GM * R));
   VR = VR - kg * VR + k * fr;
   LT = LT - kg * LT + k * fth;
   LP = LP + kg * (ygph - LP);
-  drift_f(h, X, Y, Zc, VR, LT, LP, false);
+  drift_second(h, X, Y, Zc, VR, LT, LP, r, ir, R, iR);
   x[i] = X;
   y[i] = Y;
   z[i] = Zc;

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(256) k_rad_drift(long long N, int n_inst, cons
     const double VR = vr[i], LT = lth[i], LP = lph[i];
     int cell = -1;
     if (kMixed) {
-      drift_f(h, X, Y, Zc, VR, LT, LP, true);
+      drift_first(h, X, Y, Zc, VR, LT, LP);
       mid[i] = X;
       mid[N + i] = Y;
       mid[2 * N + i] = Zc;
@@ -414,14 +414,14 @@ __global__ void __launch_bounds__(256) k_rad_kick(long long N, int n_inst, const
   if (kMixed) {
     double X = mid[i], Y = mid[N + i], Zc = mid[2 * N + i];
     const double R2 = X * X + Y * Y, R = sqrt(R2), r = sqrt(R2 + Zc * Zc);
-    const double ir = 1.0 / r, sth = R * ir, cth = Zc * ir, ir2 = ir * ir;
+    const double ir = 1.0 / r, iR = 1.0 / R, cth = Zc * ir, ir2 = ir * ir, isth = r * iR;
     float tau = 0.0f;
     if (p.tau_on)
       tau = tau_interp32(p, Tb, p.tau_geom == GD_TAU_2D ? (float)R : (float)r,
                          p.tau_geom == GD_TAU_2D ? 0.0f : (float)cth, atan2f((float)Y, (float)X));
     const float be = (float)taper * (p.f_beta0 * (p.f_rad_s0 / (float)si)) * expf(-tau);
-    const double fr = (-p.GM * (1.0 - (double)be) + LT * LT * ir + LP * LP * r / R2) * ir2;
-    const double fth = LP * LP * cth * ir2 / (sth * sth * sth);
+    const double fr = (-p.GM * (1.0 - (double)be) + LT * LT * ir + LP * LP * isth * iR) * ir2;
+    const double fth = LP * LP * cth * ir2 * (isth * isth * isth);
     // the gas disk at the midpoint in FP32, as the plain mixed step
     const float Rf = (float)R, Zf = (float)Zc;
     const float Om = sqrtf(p.f_GM / Rf) / Rf;
@@ -437,11 +437,11 @@ __global__ void __launch_bounds__(256) k_rad_kick(long long N, int n_inst, const
     const float g_r = gam + 2.0f * gpr, g_t = gam + gpr;
     const float k_r = g_r > 0.0f ? -expm1f(-(float)dt * g_r) / g_r : (float)dt;
     const float k_t = g_t > 0.0f ? -expm1f(-(float)dt * g_t) / g_t : (float)dt;
-    const double ygph = sqrt(1.0 - 2.0 * (double)eta) * sqrt(p.GM * R);
+    const double ygph = sqrt((1.0 - 2.0 * (double)eta) * (p.GM * R));
     VR = VR - (double)(k_r * g_r) * VR + (double)k_r * fr;
     LT = LT - (double)(k_t * g_t) * LT + (double)k_t * fth;
     LP = LP + (double)(k_t * gam) * (ygph - LP) - (double)(k_t * gpr) * LP;
-    drift_f(h, X, Y, Zc, VR, LT, LP, false);
+    drift_second(h, X, Y, Zc, VR, LT, LP, r, ir, R, iR);
     x[i] = X;
     y[i] = Y;
     z[i] = Zc;
