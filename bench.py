@@ -126,11 +126,11 @@ def algo_bytes(kernel, K, mixed):
 # bench command (dram__bytes_read.sum + dram__bytes_write.sum), per particle.  The records
 # hold only while the sources the measured kernels compile from (their files and the shared
 # headers) have the content they had at the capture.
-TRAFFIC_CSRC_SHA256 = "17f6a141db53d1c16b3fc20f84a8e053f924b69d711a83d178dbf65341901778"
+TRAFFIC_CSRC_SHA256 = "7ac1024b2c68cad72c6eb4548d52c0efce7faacc34e93d5dad4641de9eda1ef9"
 TRAFFIC = {
-    "knn": {"workload": "disk22", "bytes_per_particle": 253.53},
-    "rates": {"workload": "disk22", "bytes_per_particle": 190.38},
-    "sample": {"workload": "disk22", "bytes_per_particle": 117.94},
+    "knn": {"workload": "disk22", "bytes_per_particle": 253.62},
+    "rates": {"workload": "disk22", "bytes_per_particle": 190.40},
+    "sample": {"workload": "disk22", "bytes_per_particle": 149.93},
 }
 
 
@@ -141,7 +141,7 @@ INST_CSRC_SHA256 = TRAFFIC_CSRC_SHA256
 INST = {
     "knn": {"workload": "disk22", "inst": 455.79, "fp64_inst": 1.8243},
     "rates": {"workload": "disk22", "inst": 324.57, "fp64_inst": 0.18763},
-    "sample": {"workload": "disk22", "inst": 252.60, "fp64_inst": 6.4503},
+    "sample": {"workload": "disk22", "inst": 267.43, "fp64_inst": 7.0644},
 }
 
 # Issue rate of the SMs: 4 schedulers per SM, one warp instruction each per cycle.

@@ -1935,7 +1935,7 @@ __global__ void __launch_bounds__(32) k_defer_finish(McArgs A) {
 // Bound by the latency of the longest chain: of 2^22 particles of a broad disk one takes 3,408
 // events, and SMs ran out of work after 3.4 ms of 8.4.  An event's draws, logarithms and sums are
 // kept off its serial path (8.4 -> 7.8 ms alone, FP64 form of 1.5 million particles 16.7 -> 12).
-// kBlk blocks of 64 fit an SM: four leave a warp the registers to keep an event's values, six have
+// kBlk blocks of 64 fit an SM: four leave a warp the registers to keep an event's values, seven have
 // more warps to hide the chunks' loads.  Which: sample_launch.
 template <typename T, int S, int kBlk>
 __global__ void __launch_bounds__(64, kBlk) k_sample(McArgs A) {
@@ -2169,15 +2169,16 @@ static void sample_blocks(gd_ctx* c, const McArgs& A) {
 
 // Up to 2^20 particles a warp has at most some 16 chunks and the longest chain decides: four
 // blocks an SM (2^20 broad, K = 48: 2.83 ms against 3.19 with six; eight groups of 2^18: 1.4x).
-// Above, the chunks weigh more: six (2^22: an interval of three contexts at once 8.42 ms against
-// 8.72 with four).  The FP64 form fits four either way.
+// Above, the chunks weigh more: seven (2^22: an interval of three contexts at once 8.37 ms against
+// 8.53 with six; a context alone 9.32 ms a step against 9.42, and 9.59 with four).  The FP64 form
+// fits four either way.
 template <typename T, int S>
 static void sample_launch(gd_ctx* c, const McArgs& A) {
   if constexpr (sizeof(T) == 8) {
     sample_blocks<T, S, 4>(c, A);
   } else {
     if (A.N <= (1LL << 20)) sample_blocks<T, S, 4>(c, A);
-    else sample_blocks<T, S, 6>(c, A);
+    else sample_blocks<T, S, 7>(c, A);
   }
 }
 
