@@ -2,7 +2,7 @@
 """Benchmark of the collision step: particle-interval updates per second.
 
 A step is one frozen-neighbour interval of the whole hot path over every particle:
-gd_build_neighbors (cell list + K-NN), gd_collision_rates (pair rates, bin moments,
+gd_build_neighbors (order, tree + K-NN), gd_collision_rates (pair rates, bin moments,
 interval choice) and gd_sample_collisions (events, mass/weight updates, audit).
 
 Default workload: the global disk of 2^22 particles with log-normal diameters
