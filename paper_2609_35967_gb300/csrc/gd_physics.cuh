@@ -388,6 +388,16 @@ __device__ __forceinline__ void regroup64(PairOut<float>& o, double m_i, double 
   o.group64 = 0;
 }
 
+// |ln(b/a)| of two FP64 masses in FP32, over the lesser one: for a loss as for a growth the
+// argument is not negative, so log1p keeps the relative error of its argument (three roundings)
+// however large the ratio.  (Over the mass at the run's start a loss by the factor F takes the
+// argument to -1 + 1/F, whose rounding is F/ln F of the logarithm: 1.7e-5 at F = 1,600, 1e-4 at
+// 10^4, past the 2e-5 within which the audit of the mixed form looks for near ties.)
+__host__ __device__ __forceinline__ float abs_log_ratio(double a, double b) {
+  const double lo = a < b ? a : b, hi = a < b ? b : a;
+  return log1pf((float)(hi - lo) / (float)lo);
+}
+
 // J = |ln(s'/s_i)| of the deterministic channels (Sect. 2.5.3): ln(1 + N psi)/3 for
 // sticking, |ln(1 - N psi)|/3 and |ln psi|/3 for the erosion remnant and debris;
 // fragmentation uses the precomputed <J>, <J^2> of particle i.

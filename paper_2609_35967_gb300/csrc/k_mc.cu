@@ -1286,13 +1286,13 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
     unsigned h = 0u;
     // J = sum |ln s'/s| telescopes over a run of events of one direction (growth by sticking,
     // loss by erosion): one logarithm where the direction turns.  Mixed form: from the FP64
-    // masses at the run's ends, |ln(1 + (m' - m)/m)|/3 in FP32.
+    // masses at the run's ends (abs_log_ratio), a third of it, in FP32.
     T J = (T)0;
     double run = kMixed ? m : s;
     int dir = 0;
     auto flush_run = [&](double at) {
       if (dir != 0) {
-        if constexpr (kMixed) J += fabsf(log1pf(__fdiv_rn((float)(at - run), (float)run))) * (1.0f / 3.0f);
+        if constexpr (kMixed) J += abs_log_ratio(run, at) * (1.0f / 3.0f);
         else J += fabs(log(at / run));
       }
       run = at;
