@@ -232,8 +232,16 @@ template <typename T>
 __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T m_j, T Nq_j, T inv_m_j) {
   PairOut<T> o;
   const T one = (T)1;
-  T psi;
-  psi = m_j * q.inv_m;
+  T psi = m_j * q.inv_m;
+  if constexpr (sizeof(T) == 8) {
+    // The rounded quotient m_j/m_i, as the oracle has it: grains of round mass ratios (a tenth, a
+    // millionth and its parts, as equal grains grow into) lie on a threshold of psi, and the product
+    // with 1/m_i, an ulp off, decided otherwise for one such pair in twenty.  The product's exact
+    // remainder corrects it (P. Markstein, IBM J. Res. Dev. 34, 1990): 1.5 million grains 26.4 ->
+    // 26.7 ms, with a division 25.4 -> 26.3 ms in the same kind of run.
+    if (mid_range(m_j) && mid_range(q.m)) psi = fma(fma(-psi, q.m, m_j), q.inv_m, psi);
+    else psi = m_j / q.m;
+  }
   T ncoll = one;
   T vg = (T)0;      // 1e-4 / psi when grouped
   if (psi <= (T)1e-6) {
