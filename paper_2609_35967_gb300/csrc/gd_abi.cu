@@ -63,7 +63,7 @@ static cudaError_t dalloc(T** p, size_t n) {
 }
 
 static void free_all(gd_ctx* c) {
-  void* ptrs[] = {c->d_off, c->d_tile_off, c->d_inst, c->d_tree, c->d_state, c->d_bins, c->d_stile_off,
+  void* ptrs[] = {c->d_off, c->d_tile_off, c->d_tile, c->d_inst, c->d_tree, c->d_state, c->d_bins, c->d_stile_off,
                   c->d_digits, c->d_chunk, c->d_lev, c->d_node_a, c->d_node_b, c->d_perm,
                   c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64, c->d_snap32, c->d_Mr, c->d_dist, c->d_V,
                   c->d_lam, c->d_nbr, c->d_counters, c->d_sums, c->d_dprev, c->d_redo, c->d_gx,
@@ -191,12 +191,10 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
     return GD_ERR_CUDA;
   }
 
-  // Tiles of the per-particle passes: eight blocks an SM where there are particles for it.  (One
-  // block of 4096 took 203 us for the FP64 bin sums of a 4096-particle patch; with blocks of 256
-  // ten intervals of it take 2.17 ms instead of 2.89.)
-  c->tile = kTileMin;
-  while (c->tile < kTileMax && N / c->tile > 8LL * c->num_sms) c->tile *= 2;
-  std::vector<long long> tiles = tile_table(c->h_off, c->tile);
+  // tiles of the per-particle passes
+  std::vector<int> tile(n);
+  for (int b = 0; b < n; ++b) tile[b] = tile_of(c->h_off[b + 1] - c->h_off[b]);
+  std::vector<long long> tiles = tile_table(c->h_off, tile);
   c->n_tiles = (int)tiles.back();
   // units: one per spatial group of each instance
   c->h_unit0.resize(n);
@@ -208,6 +206,7 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
     if (G > 1) c->grouped = true;
   }
   c->U = (int)unit_inst.size();
+  for (int u = 0; u < c->U; ++u) tile.push_back(tile[unit_inst[u]]);
   c->n_btiles = c->grouped ? c->n_tiles + c->U : c->n_tiles;
   c->cell_cap = 16 * N + 64LL * n + 1024;
   for (int b = 0; b < n; ++b)
@@ -218,6 +217,7 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   bool ok = true;
   ok &= dalloc(&c->d_off, n + 1) == cudaSuccess;
   ok &= dalloc(&c->d_tile_off, n + 1) == cudaSuccess;
+  ok &= dalloc(&c->d_tile, tile.size()) == cudaSuccess;
   ok &= dalloc(&c->d_inst, n) == cudaSuccess;
   ok &= dalloc(&c->d_tree, n) == cudaSuccess;
   ok &= dalloc(&c->d_state, c->U) == cudaSuccess;
@@ -379,6 +379,7 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_off, c->h_off.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_tile_off, tiles.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_tile, tile.data(), sizeof(int) * tile.size(), cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_stile_off, stiles.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_tree, tree.data(), sizeof(TreeDev) * n, cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_lev, c->h_lev.data(), sizeof(int) * c->h_lev.size(), cudaMemcpyHostToDevice, str);

@@ -30,7 +30,8 @@ struct gd_ctx {
   long long* d_off = nullptr;           // [n_inst + 1]
   long long* d_tile_off = nullptr;      // [n_inst + 1] first per-particle tile of each instance
   int n_tiles = 0;
-  int tile = gd::kTileMax;              // particles per tile: see gd_create
+  int* d_tile = nullptr;                // [n_inst + U] particles per tile of each instance (tile_of),
+                                        // then of each unit (its instance's)
   gd::InstDev* d_inst = nullptr;        // [n_inst]
   gd::TreeDev* d_tree = nullptr;        // [n_inst] search trees
   gd::StateDev* d_state = nullptr;      // [n_inst]
@@ -159,7 +160,7 @@ inline TileMap tile_map(const gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_off;
   tm.n_inst = c->n_inst;
-  tm.tile = c->tile;
+  tm.tile = c->d_tile;
   tm.tile_off = c->d_tile_off;
   return tm;
 }
@@ -171,7 +172,7 @@ inline TileMap bins_map(const gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_uoff;
   tm.n_inst = c->U;
-  tm.tile = c->tile;
+  tm.tile = c->d_tile + c->n_inst;
   tm.tile_off = c->d_utile_off;
   return tm;
 }
@@ -204,7 +205,7 @@ cudaError_t launch_spectrum(gd_ctx* c);
 cudaError_t launch_outputs_knn(gd_ctx* c, int* nbr_out, double* d_out);
 cudaError_t launch_outputs_lam(gd_ctx* c, double* lam_out);
 
-std::vector<long long> tile_table(const std::vector<long long>& off, int tile);
+std::vector<long long> tile_table(const std::vector<long long>& off, const std::vector<int>& tile);
 
 // event timing around a launch (no-op unless GD_FLAG_TIMING)
 void time_begin(gd_ctx* c, int slot);

@@ -37,7 +37,8 @@ __global__ void __launch_bounds__(256) k_group_assign(TileMap tm, const InstDev*
 __global__ void k_group_scan(const InstDev* __restrict__ P, const long long* __restrict__ tile_off,
                              const int* __restrict__ unit_inst, int U, const int* __restrict__ tcount,
                              long long* __restrict__ tbase, long long* __restrict__ uoff,
-                             long long* __restrict__ utile_off, StateDev* st, long long N, int tile) {
+                             long long* __restrict__ utile_off, StateDev* st, long long N,
+                             const int* __restrict__ utile) {
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int u = threadIdx.x >> 5; u < U; u += nw) {
     const int b = unit_inst[u], g = u - P[b].unit0;
@@ -74,7 +75,7 @@ __global__ void k_group_scan(const InstDev* __restrict__ P, const long long* __r
     long long t = 0;
     for (int u = 0; u < U; ++u) {
       utile_off[u] = t;
-      t += (st[u].members + tile - 1) / tile;
+      t += (st[u].members + utile[u] - 1) / utile[u];
     }
     utile_off[U] = t;
     uoff[U] = N;
@@ -331,13 +332,15 @@ cudaError_t launch_groups(gd_ctx* c) {
   time_begin(c, 0);
   k_group_assign<<<c->n_tiles, 256, 0, c->stream>>>(tile_map(c), c->d_inst, c->x, c->y, c->d_unit_i, c->d_tcount);
   k_group_scan<<<1, 1024, 0, c->stream>>>(c->d_inst, c->d_tile_off, c->d_unit_inst, c->U, c->d_tcount, c->d_tbase,
-                                          c->d_uoff, c->d_utile_off, c->d_state, c->N, c->tile);
+                                          c->d_uoff, c->d_utile_off, c->d_state, c->N,
+                                          c->d_tile + c->n_inst);
   k_group_scatter<<<c->n_tiles, 128, 0, c->stream>>>(tile_map(c), c->d_inst, c->d_unit_i, c->d_tbase,
                                                      c->d_rank_of, c->d_gperm, c->d_unit_r);
   // the ranks by unit, for the round lists
   k_unit_count<<<c->n_tiles, 256, 0, c->stream>>>(tile_map(c), c->d_inst, c->d_unit_r, c->d_tcount);
   k_group_scan<<<1, 1024, 0, c->stream>>>(c->d_inst, c->d_tile_off, c->d_unit_inst, c->U, c->d_tcount, c->d_tbase,
-                                          c->d_uoff, c->d_utile_off, c->d_state, c->N, c->tile);
+                                          c->d_uoff, c->d_utile_off, c->d_state, c->N,
+                                          c->d_tile + c->n_inst);
   k_group_scatter<<<c->n_tiles, 128, 0, c->stream>>>(tile_map(c), c->d_inst, c->d_unit_r, c->d_tbase, nullptr,
                                                      c->d_rperm, nullptr);
   time_end(c);

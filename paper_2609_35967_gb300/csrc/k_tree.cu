@@ -627,9 +627,9 @@ namespace gd {
 
 int num_tiles(gd_ctx* c) { return c->n_tiles; }
 
-std::vector<long long> tile_table(const std::vector<long long>& off, int tile) {
+std::vector<long long> tile_table(const std::vector<long long>& off, const std::vector<int>& tile) {
   std::vector<long long> t(off.size(), 0);
-  for (size_t b = 0; b + 1 < off.size(); ++b) t[b + 1] = t[b] + (off[b + 1] - off[b] + tile - 1) / tile;
+  for (size_t b = 0; b + 1 < off.size(); ++b) t[b + 1] = t[b] + (off[b + 1] - off[b] + tile[b] - 1) / tile[b];
   return t;
 }
 
@@ -638,7 +638,7 @@ std::vector<long long> tile_table(const std::vector<long long>& off, int tile) {
 // the instances concatenated inside a level.
 std::vector<long long> tree_plan(gd_ctx* c) {
   const int n = c->n_inst;
-  const std::vector<long long> st = tile_table(c->h_off, kSortTile);
+  const std::vector<long long> st = tile_table(c->h_off, std::vector<int>(n, kSortTile));
   c->n_stiles = (int)st.back();
   c->n_chunks = (int)((256LL * c->n_stiles + kChunk - 1) / kChunk);
   long long nmax = 0;
@@ -714,7 +714,7 @@ cudaError_t launch_tree(gd_ctx* c) {
   TileMap tm;
   tm.off = c->d_off;
   tm.n_inst = c->n_inst;
-  tm.tile = kSortTile;
+  tm.tile = nullptr;                                // (kSortTile: stile_range)
   tm.tile_off = c->d_stile_off;
   const int nt = c->n_stiles;
   cudaStream_t st = c->stream;
