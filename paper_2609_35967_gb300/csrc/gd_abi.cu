@@ -212,7 +212,9 @@ extern "C" gd_status gd_create(gd_ctx** out, const gd_config* cfg) {
   for (int b = 0; b < n; ++b)
     if (cfg->params[b].cell_size > 0.0) c->check_cells = true;
   if (c->cell_factor < 1e-3) c->check_cells = true;
-  const std::vector<long long> stiles = tree_plan(c);
+  std::vector<long long> stiles(n + 1);
+  c->h_lev.resize((size_t)kMaxLev * (n + 1));
+  tree_plan(c, c->h_off.data(), c->h_lev.data(), stiles.data());
 
   bool ok = true;
   ok &= dalloc(&c->d_off, n + 1) == cudaSuccess;

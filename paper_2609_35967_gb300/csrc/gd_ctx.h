@@ -52,7 +52,8 @@ struct gd_ctx {
   int max_lev = 1;                      // levels of the deepest instance
   int* d_lev = nullptr;                 // [kMaxLev * (n_inst + 1)] first node of each instance at
                                         // each level (absolute; end entry: one past the level)
-  std::vector<int> h_lev;
+  std::vector<int> h_lev;               // its host copy, and where the plan finds it
+  const int* lev = nullptr;
   float4* d_node_a = nullptr;           // [n_nodes] box {lo x, lo y, lo z, hi x} in units
   float2* d_node_b = nullptr;           // [n_nodes] {hi y, hi z}
   int* d_perm = nullptr;                // [N] rank -> caller index
@@ -178,7 +179,7 @@ inline TileMap bins_map(const gd_ctx* c) {
 }
 
 // launchers (each returns cudaGetLastError() of its launches)
-std::vector<long long> tree_plan(gd_ctx* c);   // sort tiles and levels from the offsets
+void tree_plan(gd_ctx* c, const long long* off, int* lev, long long* stile_off);   // sort tiles and levels
 cudaError_t launch_tree(gd_ctx* c);         // Hilbert order, rank-space copies, search tree
 cudaError_t launch_knn(gd_ctx* c);
 cudaError_t knn_prepare(gd_ctx* c);

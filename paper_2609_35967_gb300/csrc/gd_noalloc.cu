@@ -4,7 +4,7 @@
 // Some callers cannot call cudaMalloc: a host program that has already reserved the
 // device's memory for its own pool (a new allocation would fail or fragment it), or a
 // latency-bound loop that cannot afford cudaMalloc's implicit device synchronisation.
-// This entry point allocates nothing.  Its scratch (the order, the tree and the
+// This entry point allocates nothing, on the device or the host.  Its scratch (the order, the tree and the
 // positions along it) lives in one file-scope __device__ array of GD_FIXED_SCRATCH_BYTES
 // bytes, which every GPU that loads the library holds until the process exits.
 // The search is the library's own (k_tree.cu, k_knn.cu) on pointers into that array: a warp per
@@ -112,15 +112,15 @@ extern "C" gd_status gd_neighbors_fixed(const double* x, const double* y, const 
   c.N = n;
   c.stream = static_cast<cudaStream_t>(stream);
   c.num_sms = sms;
-  c.h_off = {0, n};
   c.x = const_cast<double*>(x);
   c.y = const_cast<double*>(y);
   c.z = const_cast<double*>(z);
   c.lists_only = true;
   c.fix_nbr = nbr_out;
   c.fix_d = d_out;
-  const std::vector<long long> stiles = gd::tree_plan(&c);
   Tables T = {};
+  T.off[1] = n;
+  gd::tree_plan(&c, T.off, T.lev, T.stile_off);
   T.inst.geometry = params->geometry;
   T.inst.model = GD_MODEL_3D;
   T.inst.kernel_mode = GD_KERNEL_PHYSICAL;
@@ -129,14 +129,11 @@ extern "C" gd_status gd_neighbors_fixed(const double* x, const double* y, const 
   T.inst.n = n;
   T.inst.n_sg = 1;
   for (int a = 0; a < 3; ++a) { T.state.bmin[a] = ~0ull; T.state.bmax[a] = 0ull; }
-  T.off[1] = n;
-  T.stile_off[1] = stiles[1];
   for (int l = 0; l < c.max_lev; ++l) {
-    T.tree.lev_off[l] = c.h_lev[2 * l];
-    T.tree.lev_n[l] = c.h_lev[2 * l + 1] - c.h_lev[2 * l];
+    T.tree.lev_off[l] = T.lev[2 * l];
+    T.tree.lev_n[l] = T.lev[2 * l + 1] - T.lev[2 * l];
     if (T.tree.lev_n[l] > 0) T.tree.nlev = l + 1;
   }
-  for (int k = 0; k < 2 * kMaxLev; ++k) T.lev[k] = c.h_lev[k];
   Tables* dT = reinterpret_cast<Tables*>(base + kOffTables);
   c.d_inst = &dT->inst;
   c.d_state = &dT->state;

@@ -633,35 +633,39 @@ std::vector<long long> tile_table(const std::vector<long long>& off, const std::
   return t;
 }
 
-// Sizes of the sort and of the tree from the offsets: the number of passes (see sort_key), the
-// sort tiles and digit-table chunks, and the node ranges of every level, level by level with
-// the instances concatenated inside a level.
-std::vector<long long> tree_plan(gd_ctx* c) {
+static long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
+
+// Sizes of the sort and of the tree from the offsets off[n_inst + 1]: the number of passes (see
+// sort_key), the sort tiles (stile_off[n_inst + 1]) and digit-table chunks, and the node ranges of
+// every level (lev[kMaxLev * (n_inst + 1)], kept by the context), level by level with the instances
+// concatenated inside a level.  Allocates nothing: gd_neighbors_fixed plans each of its calls.
+void tree_plan(gd_ctx* c, const long long* off, int* lev, long long* stile_off) {
   const int n = c->n_inst;
-  const std::vector<long long> st = tile_table(c->h_off, std::vector<int>(n, kSortTile));
-  c->n_stiles = (int)st.back();
-  c->n_chunks = (int)((256LL * c->n_stiles + kChunk - 1) / kChunk);
   long long nmax = 0;
-  for (int b = 0; b < n; ++b) nmax = std::max(nmax, c->h_off[b + 1] - c->h_off[b]);
+  stile_off[0] = 0;
+  for (int b = 0; b < n; ++b) {
+    nmax = std::max(nmax, off[b + 1] - off[b]);
+    stile_off[b + 1] = stile_off[b] + ceil_div(off[b + 1] - off[b], kSortTile);
+  }
+  c->n_stiles = (int)stile_off[n];
+  c->n_chunks = (int)ceil_div(256LL * c->n_stiles, kChunk);
   c->sort_passes = nmax <= (1LL << 18) ? 3 : 4;
-  c->h_lev.assign((size_t)kMaxLev * (n + 1), 0);
-  std::vector<long long> cnt(n);
-  for (int b = 0; b < n; ++b) cnt[b] = (c->h_off[b + 1] - c->h_off[b] + kLeaf - 1) / kLeaf;
-  int at = 0;
+  c->lev = lev;
   c->max_lev = 1;
+  int at = 0;
   for (int l = 0; l < kMaxLev; ++l) {
-    int* tab = c->h_lev.data() + (size_t)l * (n + 1);
+    int* tab = lev + (size_t)l * (n + 1);
     for (int b = 0; b < n; ++b) {
+      long long cnt = ceil_div(off[b + 1] - off[b], kLeaf);
+      for (int k = 0; k < l; ++k) cnt = cnt > kLeaf ? ceil_div(cnt, kLeaf) : 0;
       tab[b] = at;
-      at += (int)cnt[b];
-      if (cnt[b] > 0) c->max_lev = l + 1;
-      cnt[b] = cnt[b] > kLeaf ? (cnt[b] + kLeaf - 1) / kLeaf : 0;
+      at += (int)cnt;
+      if (cnt > 0) c->max_lev = l + 1;
     }
     tab[n] = at;
     if (l == 0) c->n_leaves = at;
   }
   c->n_nodes = at;
-  return st;
 }
 
 // The sizes partners read: the live sizes, or with spatial groups each particle's size as its
@@ -743,7 +747,7 @@ cudaError_t launch_tree(gd_ctx* c) {
                              c->M, c->d_perm, c->d_rank_of, c->d_pos64, c->d_posq, c->d_snap64, c->d_snap32, c->d_Mr,
                              c->d_gx, c->d_node_a, c->d_node_b, c->d_state);
   for (int l = 1; l < c->max_lev; ++l) {
-    const int* tab = c->h_lev.data() + (size_t)l * (c->n_inst + 1);
+    const int* tab = c->lev + (size_t)l * (c->n_inst + 1);
     const int nodes = tab[c->n_inst] - tab[0];
     k_levels<<<(nodes + 7) / 8, 256, 0, st>>>(l, c->n_inst, c->d_lev, c->d_tree, c->d_node_a, c->d_node_b);
   }
