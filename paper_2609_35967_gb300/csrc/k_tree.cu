@@ -264,10 +264,49 @@ __device__ __forceinline__ void hilbert_axes(unsigned (&X)[D], int nbits) {
   for (int i = 0; i < D; ++i) X[i] ^= t;
 }
 
-// The sort key (8 passes bits): along a 3D curve of 8 or 11 bits per axis (the last bit of 33
-// dropped), a 2D curve of 12 or 16 bits per axis, or the coordinate itself (1D).  24 bits
-// resolve instances of up to 2^18 particles (64 cells per particle), 32 bits the larger ones.
-__device__ __forceinline__ unsigned sort_key(int model, const TreeDev& T, int passes, int ux, int uy, int uz) {
+// How a 3D key divides its bits: axes by descending extent; the longest is cut in 2^n1 before the
+// second has a bit, these two in 2^n2 each before the third has one, and all three in 2^n3.
+//
+// Cubes of the whole extent (n1 = n2 = 0) where they leave 16 cells per particle of the instance's
+// own box: the curve is unbroken there, and a leaf across a break has a wide box (first builds of a
+// disk of 50,001: 1.04 ms, in slabs 1.11; a patch a thousandth thick of 2^20: 0.85 and 0.90 ms).
+// Slabs first where they do not: a narrow column or a thin ring had no bits left for its short axes
+// (2^18 particles, first and next builds: a column 30 box widths tall 49 and 10.6 ms, in slabs 0.76
+// and 0.43; a ring 0.001 wide and thinner 1.4 and 0.82, in slabs 1.1 and 0.33; a box 4:1, four cells
+// per particle, 0.75 and 0.54 ms for the next builds).
+struct KeyShape {
+  int axis[3], top, n1, n2, n3;                       // top: bits of the longest axis' units
+};
+
+__device__ KeyShape key_shape(const StateDev& S, const TreeDev& T, long long n, int passes) {
+  KeyShape K;
+  int len[3];                                         // bits of the largest unit
+  const bool any = S.bmin[0] <= S.bmax[0];
+  for (int a = 0; a < 3; ++a) {
+    const double ext = any ? ord_dbl(S.bmax[a]) - T.lo[a] : 0.0;
+    len[a] = 32 - __clz((int)fmin(ext * T.inv_q, 2147483647.0));
+    K.axis[a] = a;
+  }
+  for (int k = 0; k < 3; ++k) {                       // three exchanges order three
+    const int i = k == 1 ? 1 : 0;
+    if (len[K.axis[i]] < len[K.axis[i + 1]]) { const int t = K.axis[i]; K.axis[i] = K.axis[i + 1]; K.axis[i + 1] = t; }
+  }
+  const int bits = 8 * passes;
+  K.top = len[K.axis[0]];
+  const int d1 = len[K.axis[0]] - len[K.axis[1]], d2 = len[K.axis[1]] - len[K.axis[2]];
+  const bool slabs = bits - (2 * d1 + d2) < 64 - __clzll(n - 1) + 4;   // cubes waste d1 and d1 + d2 bits
+  K.n1 = slabs ? min(d1, bits) : 0;
+  K.n2 = slabs ? min(d2, (bits - K.n1) / 2) : 0;
+  K.n3 = (bits - K.n1 - 2 * K.n2 + 2) / 3;
+  return K;
+}
+
+// The sort key (8 passes bits): along a 3D curve inside cubes (see KeyShape; what the last bit per
+// axis has too many is dropped), a 2D curve of 12 or 16 bits per axis, or the coordinate itself
+// (1D).  24 bits resolve instances of up to 2^18 particles (64 cells per particle of their box), 32
+// bits the larger ones.
+__device__ __forceinline__ unsigned sort_key(int model, const TreeDev& T, const KeyShape& K, int passes, int ux, int uy,
+                                             int uz) {
   const bool wide = passes > 3;
   if (model == GD_MODEL_R) return wide ? (unsigned)ux << 1 : (unsigned)ux >> (T.bits - 24);
   if (model != GD_MODEL_3D) {
@@ -276,11 +315,29 @@ __device__ __forceinline__ unsigned sort_key(int model, const TreeDev& T, int pa
     hilbert_axes<2>(X, nb);
     return spread2(X[0]) << 1 | spread2(X[1]);
   }
-  const int nb = wide ? 11 : 8;
-  unsigned X[3] = {(unsigned)ux >> (T.bits - nb), (unsigned)uy >> (T.bits - nb), (unsigned)uz >> (T.bits - nb)};
-  hilbert_axes<3>(X, nb);
-  const unsigned long long h = spread3(X[0]) << 2 | spread3(X[1]) << 1 | spread3(X[2]);
-  return (unsigned)(wide ? h >> 1 : h);
+  const int u[3] = {ux, uy, uz};
+  unsigned v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = (unsigned)(K.axis[k] == 0 ? u[0] : K.axis[k] == 1 ? u[1] : u[2]);
+  const int n1 = K.n1, n2 = K.n2, n3 = K.n3;
+  const int below = K.top - n1;                      // bits of a slab, then of a cube
+  unsigned long long key = n1 > 0 ? v[0] >> below : 0u;
+  if (n2 > 0) {
+    const unsigned m = (1u << n2) - 1u;
+    unsigned X[2] = {(v[0] >> (below - n2)) & m, (v[1] >> (below - n2)) & m};
+    hilbert_axes<2>(X, n2);
+    key = key << (2 * n2) | spread2(X[0]) << 1 | spread2(X[1]);
+  }
+  if (n3 > 0) {
+    const unsigned m = (1u << n3) - 1u;
+    const int s = below - n2 - n3;
+    unsigned X[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) X[k] = (s >= 0 ? v[k] >> s : v[k] << -s) & m;
+    hilbert_axes<3>(X, n3);
+    key = key << (3 * n3) | spread3(X[0]) << 2 | spread3(X[1]) << 1 | spread3(X[2]);
+  }
+  return (unsigned)(key >> (n1 + 2 * n2 + 3 * n3 - 8 * passes));
 }
 
 // Adds one tile's digit counts to the digit table (digit-major inside the instance, so that
@@ -301,6 +358,7 @@ __global__ void __launch_bounds__(256) k_keys(TileMap tm, const InstDev* __restr
                                               uint2* __restrict__ kv, int* __restrict__ digits,
                                               int* __restrict__ chunk) {
   __shared__ TreeDev T;
+  __shared__ KeyShape K;
   __shared__ int h[256];
   int b;
   long long lo, hi;
@@ -309,6 +367,7 @@ __global__ void __launch_bounds__(256) k_keys(TileMap tm, const InstDev* __restr
   h[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     make_frame(P[b], st[P[b].unit0], T);
+    K = key_shape(st[P[b].unit0], T, P[b].n, passes);
     if (blockIdx.x == tm.tile_off[b]) {
       TreeDev& G = tree[b];         // the levels' fields stay as set once
       for (int a = 0; a < 3; ++a) G.lo[a] = T.lo[a];
@@ -322,7 +381,7 @@ __global__ void __launch_bounds__(256) k_keys(TileMap tm, const InstDev* __restr
     model_pos(model, x[i], y[i], z[i], X, Y, Z);
     unsigned key = passes > 3 ? ~0u : 0xFFFFFFu;
     if (isfinite(X) && isfinite(Y) && isfinite(Z))
-      key = sort_key(model, T, passes, to_unit(T, 0, X), to_unit(T, 1, Y), to_unit(T, 2, Z));
+      key = sort_key(model, T, K, passes, to_unit(T, 0, X), to_unit(T, 1, Y), to_unit(T, 2, Z));
     kv[i] = make_uint2(key, (unsigned)i);
     atomicAdd(&h[key & 255u], 1);
   }
