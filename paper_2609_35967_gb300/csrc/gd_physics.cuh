@@ -376,6 +376,11 @@ __device__ __forceinline__ PairOut<T> pair_channels(const Query<T>& q, T s_j, T 
   return o;
 }
 
+// N_coll of a grouped pair by the FP64 form's own two quotients, for a mass change taken again from
+// the masses: the state settled later is then the state that was sampled, also where 1e-4/psi is a
+// whole number (a product with 1/m_j misses it for one round mass ratio in eight).
+__host__ __device__ __forceinline__ double count64(double m_i, double m_j) { return floor(1e-4 / (m_j / m_i)); }
+
 // Mixed form: N_coll of a grouped pair from the FP64 mass m_i and 1/m_j, the channel rates
 // recomputed with it in FP32 (N_coll rounded to FP32, half a unit more of error).  The FP64
 // form forms floor(1e-4 / (m_j / m_i)); here (1e-4 m_i) (1/m_j), within 4 units of the last place

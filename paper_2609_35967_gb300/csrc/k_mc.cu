@@ -1119,7 +1119,6 @@ __device__ __forceinline__ void event64(double rho_s, double s_min, unsigned k0,
 // change takes it from the FP64 masses again.  (Rounded to FP32 it moved a mass by up to 6e-12
 // an event, 1e-11 over a chain of 5,000.)
 constexpr float kCountF32 = 0x1p24f;
-__device__ __forceinline__ double count64(double m_i, double inv_m_j) { return floor((1e-4 * m_i) * inv_m_j); }
 
 // Heavy particles with fewer logged events than this keep the in-line FP64 replay.
 constexpr int kDeferMin = 32;
@@ -1473,7 +1472,7 @@ __device__ __forceinline__ void sample_item(const McArgs& A, const int lane, con
       double ncoll = (double)ncoll_t;
       if constexpr (kMixed) {
         if (!from_po) ncoll = nc64;
-        else if (ncoll_t >= (T)kCountF32) ncoll = count64(m, A.snap64[j].inv_m);
+        else if (ncoll_t >= (T)kCountF32) ncoll = count64(m, pj.m);
       }
       double m_new, s_new = s;
       const int way = outcome == 0 ? 1 : -1;   // of s; a fragmentation ends the run by itself
@@ -1713,13 +1712,12 @@ __global__ void __launch_bounds__(32) k_defer_chain(McArgs A) {
   for (int base = 0; base < rec.n; base += 32) {
     const int k = base + lane;
     int4 L = make_int4(0, 0, 0, 0);
-    double pm = 0.0, ps = 0.0, pi = 0.0;
+    double pm = 0.0, ps = 0.0;
     if (k < rec.n) {
       L = A.dlog[rec.lbase + k];
       const Snap64 pj = A.snap64[L.y];
       pm = pj.m;
       ps = pj.s;
-      pi = pj.inv_m;
     }
     const int cnt = min(32, rec.n - base);
     for (int i = 0; i < cnt; ++i) {
@@ -1729,9 +1727,9 @@ __global__ void __launch_bounds__(32) k_defer_chain(McArgs A) {
       Snap64 pj;
       pj.m = __shfl_sync(FULLM, pm, i);
       pj.s = __shfl_sync(FULLM, ps, i);
-      pj.inv_m = __shfl_sync(FULLM, pi, i);
+      pj.inv_m = 0.0;
       pj.N = 0.0;
-      const double nc = lw >= (int)kCountF32 ? count64(m, pj.inv_m) : (double)lw;
+      const double nc = lw >= (int)kCountF32 ? count64(m, pj.m) : (double)lw;
       if (oc == 2 && !sset) {   // a fragmentation starts from the FP64 diameter
         s = s_of_m64(P.k6, m);
         sset = 1;
