@@ -126,11 +126,11 @@ def algo_bytes(kernel, K, mixed):
 # bench command (dram__bytes_read.sum + dram__bytes_write.sum), per particle.  The records
 # hold only while the sources the measured kernels compile from (their files and the shared
 # headers) have the content they had at the capture.
-TRAFFIC_CSRC_SHA256 = "7ac1024b2c68cad72c6eb4548d52c0efce7faacc34e93d5dad4641de9eda1ef9"
+TRAFFIC_CSRC_SHA256 = "b0e9a40d4e2c37396c661f2b07371c5eb93a1b8dc2b1f204181fcc86c6b25f9f"
 TRAFFIC = {
-    "knn": {"workload": "disk22", "bytes_per_particle": 253.62},
-    "rates": {"workload": "disk22", "bytes_per_particle": 190.40},
-    "sample": {"workload": "disk22", "bytes_per_particle": 149.93},
+    "knn": {"workload": "disk22", "bytes_per_particle": 253.74},
+    "rates": {"workload": "disk22", "bytes_per_particle": 190.61},
+    "sample": {"workload": "disk22", "bytes_per_particle": 151.23},
 }
 
 
@@ -141,7 +141,7 @@ INST_CSRC_SHA256 = TRAFFIC_CSRC_SHA256
 INST = {
     "knn": {"workload": "disk22", "inst": 455.79, "fp64_inst": 1.8243},
     "rates": {"workload": "disk22", "inst": 324.57, "fp64_inst": 0.18763},
-    "sample": {"workload": "disk22", "inst": 267.43, "fp64_inst": 7.0644},
+    "sample": {"workload": "disk22", "inst": 268.93, "fp64_inst": 7.1378},
 }
 
 # Issue rate of the SMs: 4 schedulers per SM, one warp instruction each per cycle.
@@ -217,16 +217,13 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(rows)}
 
 
-def measure_form(gd, insts, dev, precision, steps, warmup, world, push=False, graph=False,
-                 cell_factor=0.0, cell_xsplit=0, timing=True):
+def measure_form(gd, insts, dev, precision, steps, warmup, world, push=False, graph=False, timing=True):
     """Times `steps` whole intervals of one form after `warmup` (CUDA events on the library's
     stream, barrier and synchronize on both sides).  graph: the intervals are replayed as a
     captured CUDA graph (gd_run_intervals), which per-kernel timing cannot see into."""
     import torch
     sess = gd.Session(insts, precision=precision, device=str(dev), velocities=push,
-                      flags=gd.GD_FLAG_TIMING if (timing and not graph) else 0, cell_factor=cell_factor,
-                      cell_xsplit=cell_xsplit)
-    cf, xs = (cell_factor, max(1, cell_xsplit)) if cell_factor > 0 else sess.autotune()
+                      flags=gd.GD_FLAG_TIMING if (timing and not graph) else 0)
     st = sess.stream
 
     def step():
@@ -262,8 +259,8 @@ def measure_form(gd, insts, dev, precision, steps, warmup, world, push=False, gr
            "kernel_ms": {k: post["kernel_ms"][k] - pre["kernel_ms"][k] for k in post["kernel_ms"]},
            "kernel_calls": {k: post["kernel_calls"][k] - pre["kernel_calls"][k]
                             for k in post["kernel_calls"]},
-           "events": post["events"] - pre["events"], "status": post["status"], "cell_factor": cf,
-           "cell_xsplit": xs, "knn_redo": post["knn_redo"] - pre["knn_redo"],
+           "events": post["events"] - pre["events"], "status": post["status"],
+           "knn_redo": post["knn_redo"] - pre["knn_redo"],
            "rate_redo": post["rate_redo"] - pre["rate_redo"],
            "sample_redo": post["sample_redo"] - pre["sample_redo"],
            "sample_deferred": post["sample_deferred"] - pre["sample_deferred"],
@@ -272,14 +269,13 @@ def measure_form(gd, insts, dev, precision, steps, warmup, world, push=False, gr
     return res
 
 
-def measure_collide(gd, insts, dev, G, steps, warmup, cell_factor, cell_xsplit):
+def measure_collide(gd, insts, dev, G, steps, warmup):
     """Whole collision steps (gd_collide over dt_coll, one neighbour build each) of the
     workload split into G spatial groups per instance, mixed form: CUDA events on the library
     stream around the timed steps (gd_collide synchronises after every round inside them)."""
     import torch
     xi = [dict(i, params=dict(i["params"], spatial_groups=G)) for i in insts]
-    sess = gd.Session(xi, precision=gd.GD_MIXED, device=str(dev), flags=gd.GD_FLAG_TIMING,
-                      cell_factor=cell_factor, cell_xsplit=cell_xsplit)
+    sess = gd.Session(xi, precision=gd.GD_MIXED, device=str(dev), flags=gd.GD_FLAG_TIMING)
     tau = insts[0]["params"]["dt_coll"]
     for _ in range(warmup):
         sess.collide(tau)
@@ -325,18 +321,16 @@ def run_gpu(args, rank, world):
     N = int(sum(len(i["x"]) for i in insts))
     hbm, peak_kind = peaks()
 
-    mixed = measure_form(gd, insts, dev, gd.GD_MIXED, args.steps, args.warmup, world, push=push,
-                         cell_factor=args.cell_factor, cell_xsplit=args.cell_xsplit)
+    mixed = measure_form(gd, insts, dev, gd.GD_MIXED, args.steps, args.warmup, world, push=push)
     fp64 = None
     if not args.skip_fp64:
         fp64 = measure_form(gd, insts, dev, gd.GD_FP64, max(1, args.steps // 3), max(1, args.warmup // 3), world,
-                            push=push, cell_factor=args.cell_factor, cell_xsplit=args.cell_xsplit)
+                            push=push)
 
     # end to end through the C ABI with host buffers: H2D of the step's inputs from
     # pinned memory and D2H of the diameters inside the timed region, every step
     cat = W.concat(insts)
-    sess = gd.Session(insts, precision=gd.GD_MIXED, device=str(dev), velocities=push,
-                      cell_factor=mixed["cell_factor"], cell_xsplit=mixed["cell_xsplit"])
+    sess = gd.Session(insts, precision=gd.GD_MIXED, device=str(dev), velocities=push)
     host = {k: torch.as_tensor(cat[k]).pin_memory() for k in ("x", "y", "z", "s", "M")}
     s_back = torch.empty(N, dtype=torch.float64).pin_memory()
     st = sess.stream
@@ -378,9 +372,7 @@ def run_gpu(args, rank, world):
             xpush, xgraph = name == "disk24", name == "patches256"
             m = measure_form(gd, xinsts, dev, gd.GD_MIXED, xsteps, xwarm, world, push=xpush, graph=xgraph)
             # the graph's per-kernel split, from a short timed run of the same intervals
-            split = (measure_form(gd, xinsts, dev, gd.GD_MIXED, 2, 1, world, push=xpush,
-                                  cell_factor=m["cell_factor"], cell_xsplit=m["cell_xsplit"])
-                     if xgraph else m)
+            split = measure_form(gd, xinsts, dev, gd.GD_MIXED, 2, 1, world, push=xpush) if xgraph else m
             f = measure_form(gd, xinsts, dev, gd.GD_FP64, 1, 1, world, push=xpush, graph=xgraph,
                              timing=False)
             t = max_over_ranks([m["ms"], f["ms"]], world, dev)
@@ -392,8 +384,7 @@ def run_gpu(args, rank, world):
     # in eight radial groups
     groups = None
     if not args.skip_extra and args.workload == "disk22":
-        groups = {f"G{G}": measure_collide(gd, insts, dev, G, 2, 1, mixed["cell_factor"], mixed["cell_xsplit"])
-                  for G in (1, 8)}
+        groups = {f"G{G}": measure_collide(gd, insts, dev, G, 2, 1) for G in (1, 8)}
 
     times = max_over_ranks([mixed["ms"], fp64["ms"] if fp64 else 0.0, e2e_ms], world, dev)
     pp = None
@@ -681,10 +672,6 @@ def main():
     ap.add_argument("--skip-cpu", action="store_true")
     ap.add_argument("--skip-extra", action="store_true",
                     help="only the main workload (no disk24 / patches256 keys)")
-    ap.add_argument("--cell-factor", type=float, default=0.0,
-                    help="cell edge factor; 0 = pick it and the x division with gd_autotune")
-    ap.add_argument("--cell-xsplit", type=int, default=0, choices=(0, 1, 2, 4),
-                    help="x division of the cell edge when --cell-factor is given (0: 1)")
     ap.add_argument("--diffusion", action="store_true",
                     help="time the dust diffusion step alone (one JSON line, 1 GPU)")
     ap.add_argument("--split-step", action="store_true",
@@ -828,9 +815,7 @@ def result_line(r, args, world):
                        l2="no flush: working set > 129 MB L2 (lists alone 4K B/particle)",
                        parallelism=("1 GPU" if world == 1 else
                                     f"instances split across {world} ranks" if "sharding" in r["cfg"] else
-                                    f"{world} independent replicas"),
-                       cell_factor=r["mixed"]["cell_factor"],
-                       cell_xsplit=r["mixed"].get("cell_xsplit", 1)),
+                                    f"{world} independent replicas")),
         "events_per_step": r["mixed"]["events"] / args.steps,
         "knn_fp64_redo_per_step": r["mixed"].get("knn_redo", 0) / args.steps,
         "mixed_fp64_settled_per_step": {"rates": r["mixed"]["rate_redo"] / args.steps,
@@ -849,7 +834,6 @@ def result_line(r, args, world):
     if r["fp64"]:
         st = max(1, args.steps // 3)
         out["fp64"] = {"value": n_job * st / (ms_fp64 * 1e-3), "ms_per_step": ms_fp64 / st,
-                       "cell_factor": r["fp64"]["cell_factor"],
                        "kernels_ms_per_step": {k: v / st for k, v in r["fp64"]["kernel_ms"].items()
                                                if v > 0 and k != "stats"}}
         out["mixed_over_fp64"] = out["value"] / out["fp64"]["value"]
@@ -871,8 +855,7 @@ def result_line(r, args, world):
             "config": dict(x["cfg"], n_particles=x["N"], K=x["K"], precision="mixed",
                            timed="one CUDA graph replay per interval (gd_run_intervals)" if x["graph"]
                            else "gd_build_neighbors, gd_collision_rates, gd_sample_collisions"
-                           + (", gd_push_staggered" if x["push"] else ""),
-                           cell_factor=x["mixed"]["cell_factor"], cell_xsplit=x["mixed"]["cell_xsplit"]),
+                           + (", gd_push_staggered" if x["push"] else "")),
             "kernels_ms_per_step": {k: w / sst for k, w in sp["kernel_ms"].items() if w > 0 and k != "stats"},
             "roofline": roofline_of(sp["kernel_ms"], sp["kernel_calls"], x["K"], x["N"], r["hbm"],
                                     r["peak_kind"], name, r.get("pipe_peaks"),

@@ -187,8 +187,11 @@ typedef struct {
   double* lph;                 /* DEVICE [N] or NULL: l_phi    (push only)    */
   void* stream;                /* cudaStream_t; NULL = legacy default stream  */
   int64_t max_events_per_interval;   /* per particle; <= 0: 65536              */
-  double cell_factor;          /* accepted as before, without effect on the search  */
-  int32_t cell_xsplit;         /* 1, 2 or 4 (0: 1), likewise                        */
+  double cell_factor;          /* of the former cell grid: no effect on the search; below
+                                  1e-3 (and > 0) it asks for more cells than a grid could
+                                  have had and is reported (GD_ST_CAPACITY) like a too
+                                  small cell_size, the lists staying exact           */
+  int32_t cell_xsplit;         /* 1, 2 or 4 (0: 1; else GD_ERR_ARG), no effect either */
   int32_t pad1;
 } gd_config;
 
@@ -517,7 +520,7 @@ const char* gd_status_string(gd_status code);
  * that has already reserved the GPU's memory for its own pool, or a
  * latency-bound loop that cannot take cudaMalloc's implicit synchronisation.
  * gd_neighbors_fixed calls no cudaMalloc, cudaFree or allocating library
- * routine.  Its scratch is one fixed device array of GD_FIXED_SCRATCH_BYTES
+ * routine, nor does it allocate host memory.  Its scratch is one fixed device array of GD_FIXED_SCRATCH_BYTES
  * bytes inside libgd.so, which every GPU that loads the library holds until
  * the process exits.
  *
@@ -525,13 +528,15 @@ const char* gd_status_string(gd_status code);
  * (FP64 keys, minimum image in a patch): nbr_out row i = i, then the K-1
  * nearest others by (d^2, index) in ascending index order; d_out[i] = distance
  * to the farthest of them.  x, y, z: DEVICE [n]; nbr_out: DEVICE int32 [n*K];
- * d_out: DEVICE [n] or NULL; params: HOST, only geometry, box_x, box_y and
- * cell_size are read; stream: cudaStream_t (NULL = legacy default stream).
+ * d_out: DEVICE [n] or NULL; params: HOST, only geometry, model, box_x and box_y
+ * are read; stream: cudaStream_t (NULL = legacy default stream).
  *
  * Limits: n <= GD_FIXED_MAX_PARTICLES (else GD_ERR_CAPACITY, nothing runs),
  * 2 <= K <= GD_FIXED_MAX_K and K <= n, params->model == GD_MODEL_3D (else
- * GD_ERR_ARG).  A query whose search finds no K-1 others within its bounded
- * number of radius growths (a non-finite coordinate) gets a row of -1 and
+ * GD_ERR_ARG).  A query that the bounded walks leave undecided (ties, particles
+ * on one point) is settled by an exact search, whatever the positions.  A
+ * particle with a non-finite coordinate is no one's neighbour; it, and every
+ * query when fewer than K-1 others are finite, gets a row of -1 and
  * d_out = -1; the call is asynchronous and still returns GD_OK, so a caller that
  * can meet such input checks row[0] >= 0 after synchronising.
  * The first call on a device looks up the array's device address with that

@@ -197,8 +197,8 @@ cudaError_t launch_snapshot(gd_ctx* c);
 cudaError_t launch_groups(gd_ctx* c);          // units, their members and d_gperm (after the cells)
 cudaError_t launch_group_inter(gd_ctx* c);     // interaction masks (after the lists)
 cudaError_t launch_round_begin(gd_ctx* c);     // the round's groups, their broadcast and snapshot
-cudaError_t launch_schedule(gd_ctx* c);
-cudaError_t launch_broadcast_snapshot(gd_ctx* c);   // the round's broadcast and its snapshot entries        // levels of the round's groups (after k_interval)
+cudaError_t launch_schedule(gd_ctx* c);        // levels of the round's groups (after k_interval)
+cudaError_t launch_broadcast_snapshot(gd_ctx* c);   // the round's broadcast and its snapshot entries
 cudaError_t launch_step_begin(gd_ctx* c, double tau, int hold);
 cudaError_t launch_step_done(gd_ctx* c, int* d_flag);
 cudaError_t launch_stats(gd_ctx* c, double* d_sums);

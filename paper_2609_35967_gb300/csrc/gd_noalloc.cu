@@ -9,7 +9,7 @@
 // bytes, which every GPU that loads the library holds until the process exits.
 // The search is the library's own (k_tree.cu, k_knn.cu) on pointers into that array: a warp per
 // query over cell rows, which it replaces, took 3.6 ms for 50,001 particles and K = 32, this
-// 1.0 ms (0.85 in the search, whose radius starts from an estimate in every call).
+// 1.1 ms (0.9 in the search, whose radius starts from an estimate in every call).
 //
 // The result is the same as gd_build_neighbors' nbr_out / d_out for a one-instance
 // FP64 context: slot 0 the particle itself, then the K-1 nearest others by (d^2, index)

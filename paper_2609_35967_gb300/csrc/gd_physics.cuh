@@ -162,7 +162,6 @@ __device__ __forceinline__ T turb_dv2(T sa, T sb, T vg2, T tre, int& regime, T& 
 __device__ __forceinline__ bool mid_range(double v) {
   return (unsigned)__double2hiint(v) - 0x39C00000u < 0x46200000u - 0x39C00000u;
 }
-__device__ __forceinline__ bool mid_range(float) { return true; }
 
 // The same over one denominator, V_t^2 = V_g^2 (add + num / den), so that the FP64 form takes one
 // quotient (an FP64 division holds the narrow FP64 pipe for ten instructions).  In the tiny

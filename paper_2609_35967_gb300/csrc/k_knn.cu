@@ -31,10 +31,11 @@
 //
 // Bound by instruction issue and the latency of dependent steps, not by HBM: 456 warp
 // instructions per particle at K = 32 (a uniform cell grid walked by each lane alone took 654,
-// with its lanes waiting for one another), 55% of the issue slots, about 510 candidates tested
-// per leaf of 32 queries.  Builds of a 2^22-particle disk, K = 32: static 5.0 -> 3.6 ms, first
+// with its lanes waiting for one another), 55% of the issue slots at 16 warps an SM (fixed latencies
+// 2.3, loads 1.7 and shared memory 1.1 stalled warps per issue), about 510 candidates tested per leaf
+// of 32 queries.  Builds of a 2^22-particle disk, K = 32: static 5.0 -> 3.6 ms, first
 // 36.6 -> 16 ms; after a push 10.8 -> 6.5 ms (2^20: 2.6 -> 1.6); K = 48 after a push 14.7 -> 8.3
-// ms.  gd_neighbors_fixed of 50,001 particles, K = 32: 3.6 -> 1.2 ms.  The code is kept
+// ms.  gd_neighbors_fixed of 50,001 particles, K = 32: 3.6 -> 1.1 ms.  The code is kept
 // small on purpose (loops not unrolled, the reduced models' volume out of line): unrolled, it
 // missed the instruction cache and the same builds took half again as long.
 #include <climits>

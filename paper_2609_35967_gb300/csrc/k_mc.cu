@@ -2165,11 +2165,17 @@ static void sample_blocks(gd_ctx* c, const McArgs& A) {
   k_sample<T, S, kBlk><<<(int)blocks, 64, 0, c->stream>>>(A);
 }
 
-// Up to 2^20 particles a warp has at most some 16 chunks and the longest chain decides: four
-// blocks an SM (2^20 broad, K = 48: 2.83 ms against 3.19 with six; eight groups of 2^18: 1.4x).
-// Above, the chunks weigh more: seven (2^22: an interval of three contexts at once 8.37 ms against
-// 8.53 with six; a context alone 9.32 ms a step against 9.42, and 9.59 with four).  The FP64 form
-// fits four either way.
+// Four blocks an SM leave the longest chain the registers, seven have more warps for the chunks.  The
+// sampler alone, ms with four and with seven blocks on 152 SMs (the heaviest grain, and so the
+// chain, varies with the draws):
+//                 2^18        2^20        1.5e6       2^21        3 2^20      2^22
+//   broad sizes   4.65 6.42   4.4  5.9    2.4  3.0    3.7  4.6    3.30 3.02   6.1  7.7
+//   equal grains  0.33 0.40   0.164 0.160 0.204 0.198 0.276 0.258 0.45 0.50   0.497 0.438
+// So up to 2^20 particles (27 chunks a warp with four blocks) four never lose; above, each wins
+// somewhere, and seven are taken for what a step of a 2^22 disk takes with other work around it (a
+// context alone 9.32 ms a step against 9.59; three contexts at once 8.37 against 8.53 with six).  N
+// is the context's, also in a round of spatial groups that visits part of it.  The FP64 form fits
+// four either way.
 template <typename T, int S>
 static void sample_launch(gd_ctx* c, const McArgs& A) {
   if constexpr (sizeof(T) == 8) {

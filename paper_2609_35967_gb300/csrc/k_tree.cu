@@ -304,7 +304,11 @@ __device__ KeyShape key_shape(const StateDev& S, const TreeDev& T, long long n, 
 // The sort key (8 passes bits): along a 3D curve inside cubes (see KeyShape; what the last bit per
 // axis has too many is dropped), a 2D curve of 12 or 16 bits per axis, or the coordinate itself
 // (1D).  24 bits resolve instances of up to 2^18 particles (64 cells per particle of their box), 32
-// bits the larger ones.
+// bits the larger ones.  Where most particles crowd a few cells of the box (far outliers, clumps a
+// ten-thousandth of it) their keys are equal, a leaf is a random part of the crowd and its queries go
+// to the exact search: 2^18 particles of a disk with one at 1000 times its radius 180 ms a build; 64
+// clumps of 2^14 324 ms first and 284 next.  (The cell grid that was before took 787 and 185 ms for
+// the clumps, and 570 ms already for 2^16 with the outlier.)
 __device__ __forceinline__ unsigned sort_key(int model, const TreeDev& T, const KeyShape& K, int passes, int ux, int uy,
                                              int uz) {
   const bool wide = passes > 3;
@@ -589,9 +593,10 @@ __global__ void k_broadcast_snapshot(const unsigned long long* __restrict__ tota
 
 // ---------------------------------------------------------------- rank-space copies and leaves
 // A warp per leaf (32 consecutive ranks of one instance): lane = rank, the caller's arrays
-// gathered, every rank-space array written coalesced, and the leaf's box.  The scatter this
-// replaces (lane = caller index, stores at random ranks in partial sectors) moved 467 B per
-// particle through DRAM for about 160.
+// gathered, every rank-space array written coalesced, and the leaf's box.  Bound by the gather:
+// doubles read at random cost a 32-byte sector each, 570 B per particle through DRAM for about 160.
+// (The scatter it replaces, lane = caller index, stored at random ranks in partial sectors: fewer
+// bytes, 467, but 0.93 ms for 2^22 particles against 0.40.)
 template <bool kMixed, bool kLists>
 __global__ void __launch_bounds__(256) k_gather(int n_leaves, int n_inst, const int* __restrict__ leaf_off,
                                                 const long long* __restrict__ off, const InstDev* __restrict__ P,
